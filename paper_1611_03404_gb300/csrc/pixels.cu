@@ -15,11 +15,11 @@
 // dE[G] are f_i times a per-(source, image) constant vector), C_m the 2x2 curvature of the
 // pixel term, w1 = iota l_E - 2 iota^2 E[G] l_V and w2 = iota^2 l_V.
 //
-// A CTA of 128 threads takes tiles (up to 128 * PPT consecutive pixels of one patch) from the
-// work queue.  Thread 0 brings each tile's patch table and pixel records into shared memory with
-// two TMA bulk copies on one mbarrier, the next tile's while the current one is evaluated.  Each
-// thread evaluates its pixels; each warp reduce-scatters the 108 per-pixel contributions so that
-// lane l keeps sums l, l+32, l+64, l+96 (4 registers, not 108).
+// A CTA takes tiles (up to 128 * PPT consecutive pixels of one patch) from the work queue.  Thread 0
+// brings each tile's patch table and pixel records into shared memory with TMA bulk copies on one
+// mbarrier, the next tile's while the current one is evaluated.  Each lane evaluates its pixels; each
+// warp reduce-scatters the 108 per-pixel contributions so that lane l holds sums l, l+32, l+64, l+96
+// (4 registers, not 108).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -138,7 +138,7 @@ __device__ __forceinline__ int feed_issue(const ProblemDev& P, TileFeed& F, int&
       constexpr uint32_t gb = (TB_FLOATS - TB_GAL) * 4u;
       mbar_expect_tx(bar, TB_VAL * 4u + gb + pb + mb);
       bulk_copy(tab, src, TB_VAL * 4u, bar);
-      bulk_copy(tab + TB_GAL, src + TB_GAL, gb, bar);
+      bulk_copy(tab + TB_VAL, src + TB_GAL, gb, bar);
     }
     bulk_copy(spix, P.pix + F.pix, pb, bar);
     bulk_copy(pm, P.patches + t.patch, mb, bar);
@@ -423,30 +423,41 @@ struct GalAcc {
   }
 };
 
-// One galaxy mixture component's contribution at pixel offset d (squares s; D0, D1, S0-S2 the
-// same numbers in both halves of a pair): value, 5 first and 15 second derivatives over v5,
+// A pixel's offset from one PSF component's mean and its squares, each twice for packed operands.
+struct PixGeo {
+  float2 D0, D1, S0, S1, S2;
+  __device__ __forceinline__ void set(float fx, float fy, const float* mu) {
+    const float d0 = fx - mu[0], d1 = fy - mu[1];
+    const float s0 = d0 * d0, s1 = 2.f * d0 * d1, s2 = d1 * d1;
+    D0 = f2(d0, d0);
+    D1 = f2(d1, d1);
+    S0 = f2(s0, s0);
+    S1 = f2(s1, s1);
+    S2 = f2(s2, s2);
+  }
+};
+
+// 2^x by the special-function unit alone, subnormal results as 0: what that leaves out is under
+// 1.2e-38, where the rate it is added to is at least the sky's.  (exp2f spends three more
+// instructions per component on those subnormals: 4 % of the kernel.)
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// One galaxy mixture component's value at a pixel (e: its table entry).
+__device__ __forceinline__ float gal_value(const float (&e)[GT_STRIDE], const PixGeo& g) {
+  const float q = fmaf(e[GT_P + 2], g.S2.x, fmaf(e[GT_P + 1], g.S1.x, e[GT_P] * g.S0.x));
+  return e[GT_W] * ex2_ftz(q * (-0.5f * LOG2E));
+}
+
+// A galaxy mixture component of value N at a pixel: value, 5 first and 15 second derivatives over v5,
 // accumulated into its family's sums.  z = P d, q = d.P.d = z.d; b_a = l_a + Q_a.s and
 // t_a = (Q_a d) for a = axis, angle, scale; the second derivatives N (z z^T - P),
 // N (z_i b_a - 2 t_a,i), N (b_a b_b + c_ab) with c_ab = l_ab + Q_ab.s.
-// Far from a narrow component its Gaussian underflows to exactly 0 (q > ~207): where that holds on
-// every lane of the warp (lanes without a pixel count as 0) the component adds exactly nothing, and
-// the warp skips its derivative terms (on the mosaic ~19 % of warp-component pairs).  All lanes of
-// the warp must be active.
-__device__ __forceinline__ void gal_component(const float* ep, float2 D0, float2 D1, float2 S0, float2 S1, float2 S2,
-                                              bool valid, GalAcc& A) {
-  float e[GT_STRIDE];
-  const float4* e4 = reinterpret_cast<const float4*>(ep);
-#pragma unroll
-  for (int w = 0; w < GT_STRIDE / 4; ++w) {
-    const float4 t4 = e4[w];
-    e[4 * w + 0] = t4.x;
-    e[4 * w + 1] = t4.y;
-    e[4 * w + 2] = t4.z;
-    e[4 * w + 3] = t4.w;
-  }
-  const float q = fmaf(e[GT_P + 2], S2.x, fmaf(e[GT_P + 1], S1.x, e[GT_P] * S0.x));
-  const float N = e[GT_W] * exp2f(q * (-0.5f * LOG2E));
-  if (__all_sync(0xffffffffu, N == 0.f || !valid)) return;
+__device__ __forceinline__ void gal_sums(const float (&e)[GT_STRIDE], const PixGeo& g, float N, GalAcc& A) {
+  const float2 D0 = g.D0, D1 = g.D1, S0 = g.S0, S1 = g.S1, S2 = g.S2;
   const float2 z = fma2(f2(e[GT_PZ], e[GT_PZ + 1]), D1, mul2(f2(e[GT_P], e[GT_P + 1]), D0));   // (z0, z1)
   // axis and angle together, scale alone
   const float2 Q0 = f2(e[GT_Q01], e[GT_Q01 + 1]), Q1 = f2(e[GT_Q01 + 2], e[GT_Q01 + 3]),
@@ -473,38 +484,72 @@ __device__ __forceinline__ void gal_component(const float* ep, float2 D0, float2
   // c_ab for the pairs (00, 01), (02, 11), (12, 22)
   float2 c[3];
 #pragma unroll
-  for (int g = 0; g < 3; ++g) {
-    const float* G = e + GT_CAB + 8 * g;
-    c[g] = fma2(f2(G[6], G[7]), S2, fma2(f2(G[4], G[5]), S1, fma2(f2(G[2], G[3]), S0, f2(G[0], G[1]))));
+  for (int h = 0; h < 3; ++h) {
+    const float* G = e + GT_CAB + 8 * h;
+    c[h] = fma2(f2(G[6], G[7]), S2, fma2(f2(G[4], G[5]), S1, fma2(f2(G[2], G[3]), S0, f2(G[0], G[1]))));
   }
   A.vv22_23 = fma2(NN, c[0], fma2(f2(Nb01.x, Nb01.x), b01, A.vv22_23));
   A.vv24_33 = fma2(NN, c[1], fma2(Nb01, f2(b2, b01.y), A.vv24_33));
   A.vv34_44 = fma2(NN, c[2], fma2(f2(Nb01.y, Nb2), f2(b2, b2), A.vv34_44));
 }
 
+// One component at a lane's pixel.  Far from a narrow component its Gaussian underflows to exactly 0
+// (q > ~175): where that holds on every lane of the warp (lanes without a pixel count as 0) the
+// component adds exactly nothing, and the warp skips its derivative terms (on the mosaic ~19 % of
+// warp-component pairs).  All lanes of the warp must be active.
+__device__ __forceinline__ void gal_component(const float* ep, const PixGeo& g, bool valid, GalAcc& A) {
+  float e[GT_STRIDE];
+  const float4* e4 = reinterpret_cast<const float4*>(ep);
+#pragma unroll
+  for (int w = 0; w < GT_STRIDE / 4; ++w) {
+    const float4 t4 = e4[w];
+    e[4 * w + 0] = t4.x;
+    e[4 * w + 1] = t4.y;
+    e[4 * w + 2] = t4.z;
+    e[4 * w + 3] = t4.w;
+  }
+  const float N = gal_value(e, g);
+  if (__all_sync(0xffffffffu, N == 0.f || !valid)) return;
+  gal_sums(e, g, N, A);
+}
+
 // ------------------------------------------------------------------------------ full kernel
-// HM: 0 all sums on the FP32 pipes; 1 / 2 the Jacobian cross-product on the tensor cores with
-// TF32 / BF16 hi+lo operands.
+// HM: 0 all sums on the FP32 pipes; 1 - 4 the Jacobian cross-product on the tensor cores (operand
+// forms above).
 // Tiles are double-buffered: the next tile's copies are issued before the current one is
 // evaluated.  (The tensor-core variants' staging area holds the 11 rows of A' and B'^T per warp;
-// the fragments' padding rows read one shared zero row, which keeps both buffers within the 48 KB
-// of static shared memory.)
+// the fragments' padding rows read one shared zero row.)
+//
+// Occupancy against registers: one rolled loop over the two galaxy families holds one family's 21 sums
+// in registers; the FP32 form keeps the other's in the warp's transpose scratch until the pixel's term,
+// and so fits 96 registers and 5 CTAs of four warps per SM (before: both families' sums live, 125
+// registers, 4 CTAs).  What bounds it then is the register file: a packed FMA on three distinct register
+// pairs issues every 3.4 cycles (two scalar ones every 2.2, but they take two slots: all-scalar and
+// mixed forms ran 1-8 % slower; two pixels per lane at 168 registers: 1 % slower, and a tile takes 4 us
+// longer).  13.5 M mosaic pixels, one value + gradient + Hessian call: 2.53 -> 2.34 ms (256-pixel tiles
+// 2.88 -> 2.23, 512-pixel 2.59 -> 2.23); a 1000-source field 559 -> 536 us.  The tensor-core forms spill
+// at 96 registers and stay at 4 CTAs (3xTF32: 3.02 -> 2.76 ms; with 5 CTAs 2.78).
+constexpr int SM_GAL = TB_VAL;                              // the galaxy entries' offset in the staged table
+constexpr int SM_TAB = SM_GAL + NGAL * GT_STRIDE;           // staged floats per table
+constexpr int GAL_FLOATS = (int)(sizeof(GalAcc) / sizeof(float));
+static_assert(GAL_FLOATS <= XP_LD, "one family's sums fit the warp's transpose scratch");
+__host__ __device__ constexpr int full_ctas_per_sm(int hm) { return hm ? 4 : 5; }
+
 template <int PPT, int HM>
-__global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
-  constexpr int NB = PPT >= 8 ? 1 : 2;   // (1024-pixel tiles: two pixel buffers would pass 48 KB)
-  __shared__ __align__(16) float tab_buf[NB][TB_FLOATS];
+__global__ void __launch_bounds__(BLOCK, full_ctas_per_sm(HM)) elbo_full_kernel(ProblemDev P) {
+  constexpr int NB = PPT >= 4 ? 1 : 2;   // (512-pixel tiles and larger: two pixel buffers would take a CTA per SM)
+  constexpr int NW = BLOCK / 32;
+  __shared__ __align__(16) float tab_buf[NB][SM_TAB];
   __shared__ __align__(16) float4 spix_buf[NB][BLOCK * PPT];
   __shared__ __align__(8) uint64_t bar[NB];
   __shared__ TileDev tmeta[NB];
   __shared__ __align__(16) PatchDev pmeta[NB];
   __shared__ __align__(16) TileFeed feed;
-  __shared__ float red[BLOCK / 32][128];
+  __shared__ float red[NW][128];
   // per-warp scratch: the tensor-core forms' staging of A' and B'^T, or the FP32 form's transposes
-  // for the reduce-scatter with 128-pixel tiles (with larger tiles the 18 KB cost a CTA per SM,
-  // more than the transposes save)
-  constexpr bool XP = HM == 0 && PPT == 1;
-  constexpr int WB = HM ? 2 * NRED * SYRK_LD : (XP ? 32 * XP_LD : 4);
-  __shared__ __align__(16) float wbuf[BLOCK / 32][WB];
+  // for the reduce-scatter
+  constexpr int WB = HM ? 2 * NRED * SYRK_LD : 32 * XP_LD;
+  __shared__ __align__(16) float wbuf[NW][WB];
   __shared__ __align__(16) float zrow[HM ? SYRK_LD : 4];
 
   __shared__ int slot;
@@ -530,59 +575,82 @@ __global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
   if (NB == 2 && tid == 0)
     slot = feed_issue(P, feed, i_next, tab_buf[b ^ 1], spix_buf[b ^ 1], &bar[b ^ 1], &tmeta[b ^ 1], &pmeta[b ^ 1]);
   if (!wait_tile(P, &bar[b], (it / NB) & 1u, &bar[b ^ (NB - 1)], ((it + 1) / NB) & 1u, NB == 2 && slot >= 0)) {
-    if (tid < NACC) P.partials[(size_t)tile * NACC + tid] = __int_as_float(0x7fc00000);
+    for (int q = tid; q < NACC; q += BLOCK) P.partials[(size_t)tile * NACC + q] = __int_as_float(0x7fc00000);
     return;
   }
   const float* tab = tab_buf[b];
   const float4* spix = spix_buf[b];
-  const TileDev t = tmeta[b];
-  const PatchDev pt = pmeta[b];
-  if (tid == 0) atomicAdd(P.counters + 0, (unsigned long long)t.count);
-  const SNConst c = *reinterpret_cast<const SNConst*>(&tab[TB_SNC]);
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  float dm[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // tensor-core M block (HM != 0)
+  const int t_start = tmeta[b].start, t_count = tmeta[b].count, pt_w = pmeta[b].w;
+  if (tid == 0) atomicAdd(P.counters + 0, (unsigned long long)t_count);
 
 #pragma unroll 1
   for (int r = 0; r < PPT; ++r) {
-    if (r * BLOCK + warp * 32 >= t.count) break;   // warp-uniform
+    if (r * BLOCK + warp * 32 >= t_count) {   // warp-uniform: no pixel of this warp from here on
+      if (r == 0) {
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) red[warp][32 * ch + lane] = 0.f;
+      }
+      break;
+    }
     const int i = r * BLOCK + tid;
-    const bool valid = i < t.count;
-    const int idx = t.start + (valid ? i : 0);
-    const int row = idx / pt.w, col = idx - row * pt.w;
+    const bool valid = i < t_count;
+    const int idx = t_start + (valid ? i : 0);
+    const int row = idx / pt_w, col = idx - row * pt_w;
     const float fx = (float)col, fy = (float)row;
-    const float4 pv = valid ? spix[i] : make_float4(0.f, 1.f, 0.f, 0.f);
 
-    // ---- profiles: star (value, d/dmu, d2/dmu2); galaxy families exp/deV over
-    //      v5 = (mu0, mu1, axis, angle, scale): value, 5 first, 15 second derivatives
-    float f0 = 0.f, f0m[2] = {0.f, 0.f}, f0mm[3] = {0.f, 0.f, 0.f};
-    GalAcc G[2];
-    G[0].zero();
-    G[1].zero();
+    // ---- galaxy families exp/deV over v5 = (mu0, mu1, axis, angle, scale): value, 5 first, 15 second
+    //      derivatives, one family at a time in a rolled loop: one copy of the component body, and
+    //      each family's accumulators stay statically indexed
+    GalAcc G0, G1;   // the exponential family's sums, the de Vaucouleurs family's
+    G1.zero();
+    float* const stash = wbuf[warp] + lane;
 #pragma unroll 1
+    for (int fam = 0; fam < 2; ++fam) {
+      if constexpr (HM == 0) {
+        if (fam) {
+          const float* g = reinterpret_cast<const float*>(&G1);
+#pragma unroll
+          for (int q = 0; q < GAL_FLOATS; ++q) stash[32 * q] = g[q];   // (read by the same lane below)
+        }
+      } else {
+        G0 = G1;   // (first round: zeros; second: the exponential family's sums)
+      }
+      G1.zero();
+      const int j0 = fam ? CELESTE_NEXP : 0, j1 = fam ? NMIX : CELESTE_NEXP;
+#pragma unroll 1
+      for (int k = 0; k < CELESTE_NPSF; ++k) {
+        PixGeo g;
+        g.set(fx, fy, &tab[TB_MU + 2 * k]);
+        const float* ep = &tab[SM_GAL + (k * NMIX + j0) * GT_STRIDE];
+#pragma unroll 1
+        for (int j = j0; j < j1; ++j, ep += GT_STRIDE) gal_component(ep, g, valid, G1);
+      }
+    }
+    if constexpr (HM == 0) {
+      float* g = reinterpret_cast<float*>(&G0);
+#pragma unroll
+      for (int q = 0; q < GAL_FLOATS; ++q) g[q] = stash[32 * q];
+      __syncwarp();   // the scratch is rewritten by the transposes below
+    }
+
+    const float4 pv = valid ? spix[i] : make_float4(0.f, 1.f, 0.f, 0.f);
+    const SNConst c = *reinterpret_cast<const SNConst*>(&tab[TB_SNC]);
+    // star profile: value, d/dmu, d2/dmu2
+    float f0 = 0.f, f0m[2] = {0.f, 0.f}, f0mm[3] = {0.f, 0.f, 0.f};
+#pragma unroll
     for (int k = 0; k < CELESTE_NPSF; ++k) {
       const float d0 = fx - tab[TB_MU + 2 * k], d1 = fy - tab[TB_MU + 2 * k + 1];
       const float s0 = d0 * d0, s1 = 2.f * d0 * d1, s2 = d1 * d1;
-      const float2 D0 = f2(d0, d0), D1 = f2(d1, d1), S0 = f2(s0, s0), S1 = f2(s1, s1), S2 = f2(s2, s2);
-      {
-        const float4 st = *reinterpret_cast<const float4*>(&tab[TB_STAR + 4 * k]);
-        const float q = fmaf(st.w, s2, fmaf(st.z, s1, st.y * s0));
-        const float N = st.x * exp2f(q * (-0.5f * LOG2E));
-        const float z0 = st.y * d0 + st.z * d1, z1 = st.z * d0 + st.w * d1;
-        f0 += N;
-        f0m[0] += N * z0;
-        f0m[1] += N * z1;
-        f0mm[0] += N * (z0 * z0 - st.y);
-        f0mm[1] += N * (z0 * z1 - st.z);
-        f0mm[2] += N * (z1 * z1 - st.w);
-      }
-      // one family at a time, rolled loops: the component body stays small enough for the
-      // instruction cache, and each family's accumulators stay statically indexed
-#pragma unroll 1
-      for (int j = 0; j < CELESTE_NEXP; ++j)
-        gal_component(&tab[TB_GAL + (k * NMIX + j) * GT_STRIDE], D0, D1, S0, S1, S2, valid, G[0]);
-#pragma unroll 1
-      for (int j = CELESTE_NEXP; j < NMIX; ++j)
-        gal_component(&tab[TB_GAL + (k * NMIX + j) * GT_STRIDE], D0, D1, S0, S1, S2, valid, G[1]);
+      const float4 st = *reinterpret_cast<const float4*>(&tab[TB_STAR + 4 * k]);
+      const float q = fmaf(st.w, s2, fmaf(st.z, s1, st.y * s0));
+      const float N = st.x * exp2f(q * (-0.5f * LOG2E));
+      const float z0 = st.y * d0 + st.z * d1, z1 = st.z * d0 + st.w * d1;
+      f0 += N;
+      f0m[0] += N * z0;
+      f0m[1] += N * z1;
+      f0mm[0] += N * (z0 * z0 - st.y);
+      f0mm[1] += N * (z0 * z1 - st.z);
+      f0mm[2] += N * (z1 * z1 - st.w);
     }
 
     // ---- galaxy profile over G6 = (mu0, mu1, dev, axis, angle, scale);  v5 index -> G6 index:
@@ -594,7 +662,7 @@ __global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
     cx.f0mm[0] = f0mm[0];
     cx.f0mm[1] = f0mm[1];
     cx.f0mm[2] = f0mm[2];
-    const float F0 = G[0].F, F1 = G[1].F;
+    const float F0 = G0.F, F1 = G1.F;
     const float dF = F1 - F0;
     cx.f1 = F0 + c.e * dF;
     cx.f1g[2] = c.e1 * dF;
@@ -602,12 +670,12 @@ __global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
 #pragma unroll
     for (int a = 0; a < 5; ++a) {
       const int ga = a < 2 ? a : a + 1;
-      cx.f1g[ga] = G[0].v(a) + c.e * (G[1].v(a) - G[0].v(a));
-      cx.f1gg[ga < 2 ? tri6(ga, 2) : tri6(2, ga)] = c.e1 * (G[1].v(a) - G[0].v(a));
+      cx.f1g[ga] = G0.v(a) + c.e * (G1.v(a) - G0.v(a));
+      cx.f1gg[ga < 2 ? tri6(ga, 2) : tri6(2, ga)] = c.e1 * (G1.v(a) - G0.v(a));
 #pragma unroll
       for (int bb = a; bb < 5; ++bb) {
         const int gb = bb < 2 ? bb : bb + 1;
-        cx.f1gg[tri6(ga, gb)] = G[0].vv(a, bb) + c.e * (G[1].vv(a, bb) - G[0].vv(a, bb));
+        cx.f1gg[tri6(ga, gb)] = G0.vv(a, bb) + c.e * (G1.vv(a, bb) - G0.vv(a, bb));
       }
     }
     const float f1 = cx.f1;
@@ -620,7 +688,7 @@ __global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
     const float E = pv.y + iota * EG;
     const float V = pv.z + iota2 * VG;
     const float x = pv.x;
-    if (valid) P.srcmom[pt.pix_off + idx] = make_float2(EG, VG);
+    if (valid) P.srcmom[pmeta[b].pix_off + t_start + i] = make_float2(EG, VG);
     const float rE = 1.f / E;
     const float rE2 = rE * rE;
     float ell;
@@ -671,34 +739,27 @@ __global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
     cx.A0w1 = cx.w1 * c.A0;
     cx.B0w2x2 = 2.f * cx.w2 * c.B0;
 
-    if constexpr (HM == 0 && XP) {
-      float v[32];
+    // the warp's sums: sum q lives in lane q % 32 of chunk q / 32; over a tile's rounds they add up in the
+    // warp's row of `red`
+    float* const rd = red[warp];
+    auto put = [&](int ch, float v) { rd[32 * ch + lane] = PPT == 1 || r == 0 ? v : rd[32 * ch + lane] + v; };
+    float v[32];
+    if constexpr (HM == 0) {
       float* T = wbuf[warp];
       fill_chunk<0>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[0] += warp_reduce_scatter32_smem(v, T, lane);
+      put(0, warp_reduce_scatter32_smem(v, T, lane));
       fill_chunk<1>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[1] += warp_reduce_scatter32_smem(v, T, lane);
+      put(1, warp_reduce_scatter32_smem(v, T, lane));
       fill_chunk<2>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[2] += warp_reduce_scatter32_smem(v, T, lane);
+      put(2, warp_reduce_scatter32_smem(v, T, lane));
       fill_chunk<3>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[3] += warp_reduce_scatter32_smem(v, T, lane);
-    } else if constexpr (HM == 0) {
-      float v[32];
-      fill_chunk<0>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[0] += warp_reduce_scatter32(v, lane);
-      fill_chunk<1>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[1] += warp_reduce_scatter32(v, lane);
-      fill_chunk<2>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[2] += warp_reduce_scatter32(v, lane);
-      fill_chunk<3>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[3] += warp_reduce_scatter32(v, lane);
+      put(3, warp_reduce_scatter32_smem(v, T, lane));
     } else {
       // chunks 0 and 1 hold every sum but the cross-product block (slots >= ACC_M = 42)
-      float v[32];
       fill_chunk<0, true>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[0] += warp_reduce_scatter32(v, lane);
+      put(0, warp_reduce_scatter32(v, lane));
       fill_chunk<1, true>(v, cx, std::make_integer_sequence<int, 32>{});
-      acc[1] += warp_reduce_scatter32(v, lane);
+      put(1, warp_reduce_scatter32(v, lane));
       float (*As)[SYRK_LD] = reinterpret_cast<float (*)[SYRK_LD]>(wbuf[warp]);
       float (*Bt)[SYRK_LD] = reinterpret_cast<float (*)[SYRK_LD]>(wbuf[warp] + NRED * SYRK_LD);
 #pragma unroll
@@ -709,33 +770,28 @@ __global__ void __launch_bounds__(BLOCK) elbo_full_kernel(ProblemDev P) {
         Bt[a][32 + lane] = cx.yV[a];
       }
       __syncwarp();
+      float dm[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
       syrk_mma<HM>(As, Bt, zrow, dm, lane);
       __syncwarp();   // the staging area is rewritten for the next 32 pixels
+      // D fragment (tile nt): rows g, g + 8; columns 8 nt + 2 t, 8 nt + 2 t + 1.  Entry (a, b) with
+      // a <= b < 11 is sum ACC_M + tri(a, b) (the block is symmetric; its upper half is kept).
+      const int g = lane >> 2, tq = lane & 3;
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int a = g + (e >> 1) * 8, bb = 8 * nt + 2 * tq + (e & 1);
+          if (a <= bb && bb < NRED) rd[ACC_M + a * NRED - a * (a - 1) / 2 + (bb - a)] = dm[nt][e];
+        }
     }
   }
 
-  // ---- combine the warps: sum q lives in lane q % 32 of chunk q / 32
-#pragma unroll
-  for (int ch = 0; ch < 4; ++ch) red[warp][32 * ch + lane] = acc[ch];
-  if constexpr (HM != 0) {
-    // D fragment (tile nt): rows g, g + 8; columns 8 nt + 2 t, 8 nt + 2 t + 1.  Entry (a, b) with
-    // a <= b < 11 is sum ACC_M + tri(a, b) (the block is symmetric; its upper half is kept).
-    __syncwarp();
-    const int g = lane >> 2, tq = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int a = g + (e >> 1) * 8, b = 8 * nt + 2 * tq + (e & 1);
-        if (a <= b && b < NRED) red[warp][ACC_M + a * NRED - a * (a - 1) / 2 + (b - a)] = dm[nt][e];
-      }
-  }
   __syncthreads();
-  if (tid < NACC) {
+  for (int q = tid; q < NACC; q += BLOCK) {
     float v = 0.f;
 #pragma unroll
-    for (int w = 0; w < BLOCK / 32; ++w) v += red[w][tid];
-    P.partials[(size_t)tile * NACC + tid] = v;
+    for (int w = 0; w < NW; ++w) v += red[w][q];
+    P.partials[(size_t)tile * NACC + q] = v;
   }
   const int next = slot;
   __syncthreads();   // this buffer, red and slot are rewritten after this point
@@ -882,7 +938,6 @@ __global__ void __launch_bounds__(BLOCK) elbo_value_kernel(ProblemDev P, int dif
 // ------------------------------------------------------------------------------ launchers
 // Persistent grids: a fixed number of CTAs per SM takes tiles from the device work queue over the
 // tile worklist, whose length is known only on the device.
-constexpr int FULL_CTAS_PER_SM = 4;    // 128 registers x 128 threads: 4 CTAs fill the register file
 constexpr int VALUE_CTAS_PER_SM = 8;
 
 cudaError_t launch_full(const ProblemDev& P, const double* theta, cudaStream_t st) {
@@ -892,30 +947,24 @@ cudaError_t launch_full(const ProblemDev& P, const double* theta, cudaStream_t s
   return launch_full_kernel(P, st);
 }
 
+template <int PPT, int HM>
+static void start_full(const ProblemDev& P, cudaStream_t st) {
+  const int g = std::max(1, std::min(P.n_tiles, P.n_sm * full_ctas_per_sm(HM)));
+  elbo_full_kernel<PPT, HM><<<g, BLOCK, 0, st>>>(P);
+}
+
 cudaError_t launch_full_kernel(const ProblemDev& P, cudaStream_t st) {
   if (P.n_tiles == 0) return cudaSuccess;
-  const int g = std::max(1, std::min(P.n_tiles, P.n_sm * FULL_CTAS_PER_SM));
-  if (P.hmode == 1) {
-    elbo_full_kernel<1, 1><<<g, BLOCK, 0, st>>>(P);   // the create call admits these only with 128-pixel tiles
-    return cudaGetLastError();
-  }
-  if (P.hmode == 2) {
-    elbo_full_kernel<1, 2><<<g, BLOCK, 0, st>>>(P);
-    return cudaGetLastError();
-  }
-  if (P.hmode == 3) {
-    elbo_full_kernel<1, 3><<<g, BLOCK, 0, st>>>(P);
-    return cudaGetLastError();
-  }
-  if (P.hmode == 4) {
-    elbo_full_kernel<1, 4><<<g, BLOCK, 0, st>>>(P);
-    return cudaGetLastError();
-  }
-  switch (P.tile_pixels) {
-    case 128: elbo_full_kernel<1, 0><<<g, BLOCK, 0, st>>>(P); break;
-    case 256: elbo_full_kernel<2, 0><<<g, BLOCK, 0, st>>>(P); break;
-    case 512: elbo_full_kernel<4, 0><<<g, BLOCK, 0, st>>>(P); break;
-    default: elbo_full_kernel<8, 0><<<g, BLOCK, 0, st>>>(P); break;
+  // (the create call admits the tensor-core forms only with 128-pixel tiles)
+  switch (P.hmode ? P.hmode : P.tile_pixels) {
+    case 1: start_full<1, 1>(P, st); break;
+    case 2: start_full<1, 2>(P, st); break;
+    case 3: start_full<1, 3>(P, st); break;
+    case 4: start_full<1, 4>(P, st); break;
+    case 128: start_full<1, 0>(P, st); break;
+    case 256: start_full<2, 0>(P, st); break;
+    case 512: start_full<4, 0>(P, st); break;
+    default: start_full<8, 0>(P, st); break;
   }
   return cudaGetLastError();
 }
