@@ -103,6 +103,8 @@ constexpr int WL_INTS = 8;
 // Doubles per source kept by the trust-region step for a repeated subproblem (Householder
 // vectors, tridiagonal form, reflected gradient, reflection coefficients, squared off-diagonal).
 constexpr int TR_CACHE = NP * NP + 5 * NP;
+// Doubles of the multiplier searches' factor tables (one per problem).
+constexpr int TR_FACTORS = 640;
 
 // Device view of a bound problem (passed by value to kernels).
 struct ProblemDev {

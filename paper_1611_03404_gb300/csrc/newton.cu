@@ -18,6 +18,7 @@
 
 namespace celeste {
 
+static_assert(32 * TR_FAC + 128 * TR_FAC_Q <= TR_FACTORS, "the workspace holds both searches' factors");
 constexpr int TR_WARPS = 1;     // sources per CTA of the step kernel (one warp: 29 KB of shared memory)
 
 // Per-source integer state (ST_STRIDE ints).  ST_SAME: the last step was rejected, so the next
@@ -39,6 +40,7 @@ struct NewtonDev {
   int* state;           // [S][ST_STRIDE]
   int* count;           // [0]: active sources after the update
   int* list;            // [S]: the active sources after the update (count[0] of them, any order)
+  double* fac;          // [TR_FACTORS] the multiplier searches' factors: one-warp, then four-warp
   int cta_max;          // at most this many active sources: four warps per subproblem
   int S;
   double ftol, gtol, delta0, delta_max, eta, delta_min;
@@ -57,6 +59,8 @@ __device__ inline double warp_max(double v) {
 
 __global__ void newton_init_kernel(NewtonDev N, int* flags) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < 128) tr_fac_q(s, N.fac + 32 * TR_FAC);   // (blocks of 128 threads)
+  if (s < 32) tr_fac_lane(s, N.fac);
   if (s >= N.S) return;
   N.state[ST_STRIDE * s + ST_ACTIVE] = 1;
   N.state[ST_STRIDE * s + ST_ITERS] = 0;
@@ -71,7 +75,9 @@ __global__ void newton_init_kernel(NewtonDev N, int* flags) {
   flags[s] = FLAG_FULL;
 }
 
-// One warp per source: convergence tests, subproblem, trial point.
+// One warp per source: convergence tests, subproblem, trial point.  Bound by the float64 issue of the
+// SM's four sub-partitions; 1000 field sources: 264 us per launch, 317 with a row of every update to a
+// lane and float64 comparisons.
 __global__ void __launch_bounds__(32 * TR_WARPS) tr_step_kernel(NewtonDev N, int* flags) {
   __shared__ TrSmem sm[TR_WARPS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -122,7 +128,7 @@ __global__ void __launch_bounds__(32 * TR_WARPS) tr_step_kernel(NewtonDev N, int
   double* cache = N.tcache + (size_t)s * TR_CACHE;
   double lam;
   const bool reduced = tr_solve_warp(S, HL, -1.0, gk, delta, try_newton, use_cache ? cache : nullptr, cache,
-                                     N.lam[s], lam, pk, pred, hard);
+                                     N.lam[s], N.fac, lam, pk, pred, hard);
   if (lane == 0) {
     st[ST_CACHED] = use_cache || reduced;
     N.lam[s] = lam;
@@ -189,7 +195,7 @@ __global__ void __launch_bounds__(128, 2) tr_step_cta_kernel(NewtonDev N, int* f
     // (every thread has read the source's state before the solver's first barrier; warp 0
     // writes it back below)
     const bool reduced = tr_solve_q(S, HL, -1.0, gk, delta, try_newton, use_cache ? cache : nullptr, cache,
-                                    N.lam[s], lam, pk, pred, hard);
+                                    N.lam[s], N.fac + 32 * TR_FAC, lam, pk, pred, hard);
     if (w == 0) {
       const double pnorm = sqrt(warp_sum(lane < NP ? pk * pk : 0.0));
       if (lane < NP) N.trial[(size_t)s * NP + lane] = N.theta[(size_t)s * NP + lane] + pk;
@@ -219,15 +225,17 @@ __global__ void __launch_bounds__(32 * TR_WARPS) tr_solve_batch_kernel(const dou
                                                                        const double* __restrict__ hint, double* p,
                                                                        double* pred, int* hard, double* lam_out) {
   __shared__ TrSmem sm[TR_WARPS];
+  __shared__ double fac[TR_WARPS][32 * TR_FAC];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * TR_WARPS + warp;
   if (q >= n) return;
+  tr_fac_lane(lane, fac[warp]);   // (each lane reads its own entries)
   TrSmem& S = sm[warp];
   const double gk = lane < NP ? g[(size_t)q * NP + lane] : 0.0;
   double pk, pr, lam;
   int hc;
-  tr_solve_warp(S, B + (size_t)q * NP * NP, 1.0, gk, delta[q], true, nullptr, nullptr, hint ? hint[q] : -1.0, lam,
-                pk, pr, hc);
+  tr_solve_warp(S, B + (size_t)q * NP * NP, 1.0, gk, delta[q], true, nullptr, nullptr, hint ? hint[q] : -1.0,
+                fac[warp], lam, pk, pr, hc);
   if (lane < NP) p[(size_t)q * NP + lane] = pk;
   if (lane == 0) {
     if (pred) pred[q] = pr;
@@ -244,13 +252,15 @@ __global__ void __launch_bounds__(128, 2) tr_solve_batch_cta_kernel(const double
                                                                    double* pred, int* hard, double* lam_out) {
   extern __shared__ __align__(16) unsigned char tr_cta_smem[];
   TrSmemQ& S = *reinterpret_cast<TrSmemQ*>(tr_cta_smem);
+  __shared__ double fac[128 * TR_FAC_Q];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  tr_fac_q(threadIdx.x, fac);   // (each thread reads its own entries)
   for (int q = blockIdx.x; q < n; q += gridDim.x) {
     const double gk = lane < NP ? g[(size_t)q * NP + lane] : 0.0;
     double pk = 0.0, pr = 0.0, lam = -1.0;
     int hc = 0;
-    tr_solve_q(S, B + (size_t)q * NP * NP, 1.0, gk, delta[q], true, nullptr, nullptr, hint ? hint[q] : -1.0, lam, pk,
-               pr, hc);
+    tr_solve_q(S, B + (size_t)q * NP * NP, 1.0, gk, delta[q], true, nullptr, nullptr, hint ? hint[q] : -1.0, fac,
+               lam, pk, pr, hc);
     if (w == 0) {
       if (lane < NP) p[(size_t)q * NP + lane] = pk;
       if (lane == 0) {
@@ -405,6 +415,7 @@ extern "C" int celeste_newton_batch(celeste_problem* p, double* theta, const cel
   N.count = reinterpret_cast<int*>(p->base + L.nt_count);
   N.lam = reinterpret_cast<double*>(p->base + L.nt_lam);
   N.list = reinterpret_cast<int*>(p->base + L.nt_list);
+  N.fac = reinterpret_cast<double*>(p->base + L.nt_fac);
   N.cta_max = o.cta_sources > 0 ? o.cta_sources : (o.cta_sources == 0 ? 2 * p->dev.n_sm : -1);
   N.S = p->S;
   N.ftol = o.ftol > 0 ? o.ftol : 1e-8;

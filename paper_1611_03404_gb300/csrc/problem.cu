@@ -333,6 +333,7 @@ void build_layout(celeste_problem* p) {
   L.nt_count = take(sizeof(int) * 4);
   L.nt_lam = take(sizeof(double) * S);
   L.nt_list = take(sizeof(int) * S);
+  L.nt_fac = take(sizeof(double) * TR_FACTORS);
   L.total = o;
 }
 

@@ -24,7 +24,12 @@
 //   * hard case (the bracket closes on the pole with |p| < delta): eigenvector of lambda_min by
 //     inverse iteration on T after a float32 Sturm bracket, p = y + tau z;
 //   * lane-dependent choices are selects and every lane finishes its evaluation, so the warp
-//     stays converged through the float64 passes (a split warp issues them once per part).
+//     stays converged through the float64 passes (a split warp issues them once per part);
+//   * a float64 warp instruction holds its sub-partition's pipe for 64 cycles (76 when all four of an SM
+//     issue them), comparisons included, whatever its active lanes: the rank-one and rank-two updates
+//     deal the trailing block's entries to the lanes one by one instead of a row to a lane (at 26 rows
+//     22 instructions instead of 26, at 13 six instead of 13), signs and minima are taken on the
+//     integer units, and the derivative of the secular function is formed only for a pass that needs it.
 // The step is mapped back with the reflections, p = Q y.
 #pragma once
 
@@ -69,10 +74,30 @@ __device__ __forceinline__ double tr_rcp(double a) {
   return fma(r, e, r);
 }
 
+// x > 0 (false for NaN) on the integer units: +0 < bits <= +inf.
+__device__ __forceinline__ bool tr_positive(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ULL;
+}
+
+// Doubles as integers of the same order (and back: the map is its own inverse).
+__device__ __forceinline__ long long tr_order(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffLL); }
+
 __device__ inline double tr_warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// The warp sums of a and of b: the first exchange leaves a's halves in lanes 0-15 and b's in 16-31, so
+// that both take one addition per level (the same pairs as in tr_warp_sum: additions commute).
+__device__ inline void tr_warp_sum2(double& a, double& b, int lane) {
+  const bool up = (lane & 16) != 0;
+  const double send = up ? a : b;
+  double x = (up ? b : a) + __shfl_xor_sync(0xffffffffu, send, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  a = __shfl_sync(0xffffffffu, x, 0);
+  b = __shfl_sync(0xffffffffu, x, 16);
 }
 
 // LDL^T of T + lambda I into S.D (reciprocal pivots), S.L; returns false if a pivot is not positive.
@@ -132,16 +157,14 @@ __device__ inline int tr_sturm_f(const SM& S, float x) {
 }
 
 // Lane-private evaluation at the lane's own multiplier lam: L D L^T = T + lam I (reciprocal
-// pivots in PR), y = -(T + lam I)^-1 gh in PY (PL, PR, PY: the warp's [TR_N][32] scratch); returns
-// false if a pivot is not positive.
-// Otherwise pn = |y| and qn2 = y^T (T + lam I)^-1 y (phi'(lam) = qn2 / pn^3 for
-// phi = 1/|y| - 1/delta).  All lanes run the same instruction stream on their own lam, so a pass
-// costs one evaluation's float64 instructions for 32 multipliers.
+// pivots in PR), y = -(T + lam I)^-1 gh in PY, pn = |y| (PL, PR, PY: the warp's [TR_N][32] scratch);
+// returns false if a pivot is not positive.  All lanes run the same instruction stream on their own
+// lam, so a pass costs one evaluation's float64 instructions for 32 multipliers.
 template <class SM>
 __device__ inline bool tr_eval_lane(const SM& S, double (*PL)[32], double (*PR)[32], double (*PY)[32], int lane,
-                                    double lam, double& pn, double& qn2) {
+                                    double lam, double& pn) {
   double Dp = S.d[0] + lam;
-  bool pd = Dp > 0.0;
+  bool pd = tr_positive(Dp);
   double r = tr_rcp(Dp);
   double w = -S.gh[0];
   PR[0][lane] = r;
@@ -149,7 +172,7 @@ __device__ inline bool tr_eval_lane(const SM& S, double (*PL)[32], double (*PR)[
   for (int i = 1; i < TR_N; ++i) {
     const double l = S.off[i] * r;
     Dp = fma(-S.o2[i], r, S.d[i] + lam);
-    pd = pd && Dp > 0.0;
+    pd = pd && tr_positive(Dp);
     r = tr_rcp(Dp);
     w = fma(-l, w, -S.gh[i]);
     PL[i][lane] = l;
@@ -165,25 +188,50 @@ __device__ inline bool tr_eval_lane(const SM& S, double (*PL)[32], double (*PR)[
     PY[i][lane] = y;
     p2 = fma(y, y, p2);
   }
+  pn = sqrt(p2);
+  return pd;
+}
+
+// y^T (T + lam I)^-1 y of the lane's last evaluation: phi'(lam) = that / |y|^3 for phi = 1/|y| - 1/delta.
+__device__ inline double tr_q2_lane(double (*PL)[32], double (*PR)[32], double (*PY)[32], int lane) {
   double z = PY[0][lane], q2 = z * z * PR[0][lane];
   for (int i = 1; i < TR_N; ++i) {
     z = fma(-PL[i][lane], z, PY[i][lane]);
     q2 = fma(z * z, PR[i][lane], q2);
   }
-  pn = sqrt(p2);
-  qn2 = q2;
-  return pd;
+  return q2;
 }
 
+// The one-warp search's lane factors that cost float64 instructions (TR_FAC per lane, at fac[lane + 32 q]:
+// gfac, ufac, hfac of tr_lambda_parallel), formed once per batch of solves.
+constexpr int TR_FAC = 3;
+__device__ inline void tr_fac_lane(int lane, double* fac) {
+  fac[lane] = lane < 16 ? ldexp(1.0, -3 * (16 - lane)) : (double)(lane - 15) / 17.0;
+  fac[lane + 32] = (double)(lane - 1) / 23.0;
+  fac[lane + 64] = exp2(0.5 * (double)(lane - 16) + 0.25);   // 2^-7.75 .. 2^7.75 around the hint
+}
+
+// 2^e for a normal result.
+__device__ __forceinline__ double tr_pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+
+// Warp maximum and minimum (no NaN among the values), compared on the integer units.
 __device__ inline double tr_warp_max(double v) {
+  long long k = tr_order(__double_as_longlong(v));
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long t = __shfl_xor_sync(0xffffffffu, k, o);
+    k = t > k ? t : k;
+  }
+  return __longlong_as_double(tr_order(k));
 }
 __device__ inline double tr_warp_min(double v) {
+  long long k = tr_order(__double_as_longlong(v));
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long t = __shfl_xor_sync(0xffffffffu, k, o);
+    k = t < k ? t : k;
+  }
+  return __longlong_as_double(tr_order(k));
 }
 
 // Copies lane src's y into S.y (lanes < 27 in parallel).
@@ -206,8 +254,9 @@ __device__ inline void tr_take_y(TrSmem& S, int lane, int src) {
 // its multiplier; returns 1 for the hard case (the bracket closes on the pole with phi > 0 to its
 // right), in which S.y is not set.
 __device__ inline int tr_lambda_parallel(TrSmem& S, int lane, double lo, double hi, double delta, bool try_zero,
-                                         double spec, double hint, double& lam_out) {
+                                         double spec, double hint, const double* fac, double& lam_out) {
   constexpr double TOL = 1e-10;
+  const double rdelta = tr_rcp(delta);
   double L = lo, H = hi;            // L <= lambda* <= H
   bool have_h = false;              // S.y holds the point H (phi(H) >= 0)
   double lamN = -1.0;               // Newton point from the best left evaluation (< 0: none)
@@ -223,11 +272,9 @@ __device__ inline int tr_lambda_parallel(TrSmem& S, int lane, double lo, double 
   // (the bracket shrinks at least 23-fold), lanes 24-27 above the secant point and 28-31 below
   // the Newton point at 2^-4 .. 2^-16 of the distance to the bracket's ends (in case rounding
   // has moved either across the root).
-  const double gfac = lane < 16 ? ldexp(1.0, -3 * (16 - lane)) : (double)(lane - 15) / 17.0;
-  const double nfac = ldexp(1.0, -3 * ((lane & 15) + 1));
-  const double ufac = (double)(lane - 1) / 23.0;
-  const double afac = ldexp(1.0, -4 * ((lane & 3) + 1));
-  const double hfac = exp2(0.5 * (double)(lane - 16) + 0.25);   // 2^-7.75 .. 2^7.75 around the hint
+  const double gfac = fac[lane], ufac = fac[lane + 32], hfac = fac[lane + 64];
+  const double nfac = tr_pow2(-3 * ((lane & 15) + 1));
+  const double afac = tr_pow2(-4 * ((lane & 3) + 1));
   double lamH = H;                  // multiplier of the point H
   for (int pass = 0; pass < 16; ++pass) {
     // ---- this lane's multiplier
@@ -248,8 +295,8 @@ __device__ inline int tr_lambda_parallel(TrSmem& S, int lane, double lo, double 
       if (lh > L && lh < H) lam = lh;   // else the lane keeps its bracket point
     }
     __syncwarp();   // (lane choices are selects; the evaluation below must issue once, converged)
-    double pn = 0.0, qn2 = 0.0;
-    const bool pd = tr_eval_lane(S, S.PL, S.PR, S.PY, lane, lam, pn, qn2);
+    double pn = 0.0;
+    const bool pd = tr_eval_lane(S, S.PL, S.PR, S.PY, lane, lam, pn);
     // ---- interior solution
     if (pass == 0 && try_zero) {
       const bool interior = __shfl_sync(0xffffffffu, (int)(pd && pn <= delta), 0) != 0;
@@ -277,7 +324,7 @@ __device__ inline int tr_lambda_parallel(TrSmem& S, int lane, double lo, double 
       tr_take_y(S, lane, __ffs(m) - 1);
       H = newH;
       lamH = newH;
-      phiH = tr_rcp(__shfl_sync(0xffffffffu, pn, __ffs(m) - 1)) - tr_rcp(delta);
+      phiH = tr_rcp(__shfl_sync(0xffffffffu, pn, __ffs(m) - 1)) - rdelta;
       have_h = true;
     }
     L = fmax(L, newL);
@@ -287,9 +334,10 @@ __device__ inline int tr_lambda_parallel(TrSmem& S, int lane, double lo, double 
     if (lbest > lamL) {
       const unsigned m = __ballot_sync(0xffffffffu, lft && lam == lbest);
       const int src = __ffs(m) - 1;
-      const double pnb = __shfl_sync(0xffffffffu, pn, src), qb = __shfl_sync(0xffffffffu, qn2, src);
+      const double pnb = __shfl_sync(0xffffffffu, pn, src);
+      const double qb = __shfl_sync(0xffffffffu, tr_q2_lane(S.PL, S.PR, S.PY, lane), src);
       lamL = lbest;
-      phiL = tr_rcp(pnb) - tr_rcp(delta);
+      phiL = tr_rcp(pnb) - rdelta;
       dphiL = qb * tr_rcp(pnb * pnb * pnb);
     }
     lamN = lamL > -INFINITY ? lamL - phiL * tr_rcp(dphiL) : -1.0;
@@ -319,25 +367,48 @@ __device__ inline void tr_load(TrSmem& S, const double* __restrict__ B, double b
   __syncwarp();
 }
 
-// Newton step p = -B^-1 g by L D L^T of S.A in place (lane i owns row i; the rows are kept full,
-// so row k holds the current a_kj when step k needs it).  Returns false if a pivot is not
-// positive; otherwise lane i < 27 holds p_i.
+// The lanes' walk over the m x m trailing block that starts at (k + 1, k + 1), row by row: entry e of the
+// block is (k + 1 + e / m, k + 1 + e % m), lane l of n takes e = l, l + n, ...  (i, j): offsets in the block.
+struct TrWalk {
+  int i, j, di, dj, m;
+  __device__ __forceinline__ TrWalk(int first, int n, int m_) : m(m_) {
+    i = first / m, j = first - i * m;
+    di = n / m, dj = n - di * m;
+  }
+  __device__ __forceinline__ void next() {
+    i += di;
+    j += dj;
+    if (j >= m) {
+      j -= m;
+      ++i;
+    }
+  }
+};
+
+// Newton step p = -B^-1 g by L D L^T of S.A in place (the whole trailing block is kept current, so row
+// k holds the current a_kj when step k needs it).  Returns false if a pivot is not positive; otherwise
+// lane i < 27 holds p_i.
 __device__ inline bool tr_newton_step(TrSmem& S, double gi, double& p_i) {
   const int lane = threadIdx.x & 31;
   const bool row = lane < TR_N;
   double* ar = S.A + lane * TR_LD;
   for (int k = 0; k < TR_N; ++k) {
     const double dk = S.A[k * TR_LD + k];
-    if (!(dk > 0.0)) return false;   // same value in every lane
+    if (!tr_positive(dk)) return false;   // same value in every lane
     const double r = tr_rcp(dk);
-    const bool act = row && lane > k;
-    const double li = act ? ar[k] * r : 0.0;
-    __syncwarp();
-    if (act) {
-      for (int j = k + 1; j < TR_N; ++j) ar[j] = fma(-li, S.A[k * TR_LD + j], ar[j]);
+    if (row && lane > k) {
+      const double li = ar[k] * r;
+      S.v[lane] = li;
       ar[k] = li;   // L below the diagonal
     }
     if (lane == k) S.D[k] = r;
+    __syncwarp();
+    const int m = TR_N - 1 - k;
+    if (m > 0) {
+      const double *l = S.v + k + 1, *rk = S.A + k * TR_LD + k + 1;
+      double* T = S.A + (k + 1) * TR_LD + k + 1;
+      for (TrWalk q(lane, 32, m); q.i < m; q.next()) T[q.i * TR_LD + q.j] = fma(-l[q.i], rk[q.j], T[q.i * TR_LD + q.j]);
+    }
     __syncwarp();
   }
   // L y = -g (column by column), y *= D^-1, L^T x = y (from the bottom)
@@ -360,12 +431,12 @@ __device__ inline bool tr_newton_step(TrSmem& S, double gi, double& p_i) {
 // hard case taken.  try_newton: attempt the Newton step first.  cache_in (or null): the
 // tridiagonal form of this same B and g, stored by an earlier call, replaces the reduction;
 // cache_out (or null): where to store the reduction when one is made.  lam_hint: the multiplier
-// of this source's previous subproblem (negative: none); lam_out: this one's (0 for an interior
-// step, negative after the hard case).  Returns true when the reduction was made and stored.
+// of this source's previous subproblem (negative: none); fac: the table of tr_fac_lane; lam_out: this
+// one's (0 for an interior step, negative after the hard case).  Returns true when the reduction was made and stored.
 __device__ inline bool tr_solve_warp(TrSmem& S, const double* __restrict__ Bsrc, double bsign, double gi,
                                      double delta, bool try_newton, const double* __restrict__ cache_in,
-                                     double* __restrict__ cache_out, double lam_hint, double& lam_out,
-                                     double& p_i, double& pred, int& hard) {
+                                     double* __restrict__ cache_out, double lam_hint, const double* fac,
+                                     double& lam_out, double& p_i, double& pred, int& hard) {
   const int lane = threadIdx.x & 31;
   const int n = TR_N;
   const bool row = lane < n;
@@ -432,20 +503,21 @@ __device__ inline bool tr_solve_warp(TrSmem& S, const double* __restrict__ Bsrc,
     }
     const double pi = beta * ((u[0] + u[1]) + (u[2] + u[3]));
     double vp = vi * pi, vg = vi * gh;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      vp += __shfl_xor_sync(0xffffffffu, vp, o);
-      vg += __shfl_xor_sync(0xffffffffu, vg, o);
-    }
+    tr_warp_sum2(vp, vg, lane);
     const double K = 0.5 * beta * vp;
     const double wi = pi - K * vi;
     gh = fma(-beta * vg, vi, gh);
     S.w[lane] = wi;
+    if (lane > k && row) S.A[lane * TR_LD + k] = vi;   // keep the reflection vector
     __syncwarp();
-    if (lane > k && row) {
-      double* ar = S.A + lane * TR_LD;
-      for (int j = k + 1; j < n; ++j) ar[j] = fma(-vi, S.w[j], fma(-wi, S.v[j], ar[j]));
-      ar[k] = vi;   // keep the reflection vector
+    {
+      const int m = n - 1 - k;
+      const double *v = S.v + k + 1, *w = S.w + k + 1;
+      double* T = S.A + (k + 1) * TR_LD + k + 1;
+      for (TrWalk q(lane, 32, m); q.i < m; q.next()) {
+        double* t = T + q.i * TR_LD + q.j;
+        *t = fma(-v[q.i], w[q.j], fma(-w[q.i], v[q.j], *t));
+      }
     }
     if (lane == 0) {
       S.beta[k] = beta;
@@ -494,7 +566,7 @@ __device__ inline bool tr_solve_warp(TrSmem& S, const double* __restrict__ Bsrc,
   if (lane == 0) S.flag[2] = 0;
   __syncwarp();
   lam_out = -1.0;
-  if (tr_lambda_parallel(S, lane, lo, hi, delta, lo == 0.0, spec, lam_hint, lam_out)) {
+  if (tr_lambda_parallel(S, lane, lo, hi, delta, lo == 0.0, spec, lam_hint, fac, lam_out)) {
     lam_out = -1.0;
     // hard case: g has (almost) no component along the eigenvector z of lambda_min.  lambda_min
     // from a float32 Sturm bracket refined by inverse iteration (lane 0), then

@@ -5,18 +5,23 @@
 // A warp's float64 instruction stream is what bounds one subproblem on this part (an SM
 // sub-partition retires a float64 warp instruction only every few tens of cycles), so when fewer
 // subproblems than SMs are in flight, three of every four float64 pipes idle under the one-warp
-// solver.  Here:
-//   * the L D L^T factorisation and the Householder reduction split the matrix by columns, column j
-//     belonging to warp j mod 4 (each warp updates and multiplies its own columns for every row,
-//     lane i owning row i); the scalars of a step (norms, reflection coefficients, the reductions
-//     of v.p and v.g) are formed by every warp from the same data in the same order, so all warps
-//     hold the same values, and two CTA barriers per step order the partial products and the next
-//     column;
+// solver.  Here one step's serial part runs on warp 0 while the others do what does not wait for it
+// (an SM issues one float64 warp instruction per 64 cycles and sub-partition, per 76 when all four
+// issue, and a CTA barrier costs 25; every warp repeating the serial part would only slow it down):
+//   * L D L^T: warp 0 updates column k + 1 first, and forms the next pivot's reciprocal and factors while
+//     warps 1-3 update the rest of the trailing block, its entries dealt to their lanes one by one;
+//   * Householder reduction: likewise warp 0 forms the next column's norm and reflection during the
+//     rank-two update; the product A v is split over the warps by columns (column j: warp j mod 4), and
+//     warp 1 reflects g while warp 0 forms w;
 //   * the multiplier search evaluates 128 multipliers per pass (32 per warp, lane-private
 //     recurrences on the tridiagonal form), the warps' minima and maxima combined through shared
-//     memory in a fixed order;
+//     memory in a fixed order; the derivative of the secular function is formed by the one warp whose
+//     multiplier the next pass starts from;
 //   * the hard case and the back-transformation run on warp 0 as in the one-warp solver.
 // Every branch that contains a barrier depends only on values all threads hold identically.
+// A single-source solve (20 subproblems, launches timed one by one, caches cold): 120 -> 100 us on average;
+// now 25 us for an interior Newton step, ~128 us for a reduction and three multiplier passes, 78 us
+// where the reduction is cached.
 #pragma once
 
 #include "trsolve.cuh"
@@ -26,49 +31,80 @@ namespace celeste {
 struct TrSmemQ {
   double A[TR_N * TR_LD];         // B; its L D L^T factors, or the Householder vectors below the diagonal
   double beta[TR_N];
-  double v[4][32], w[4][32];      // per-warp copies of the reflection vector and of w
+  double v[2][32];                // a step's column factors or reflection vector, by the step's parity
+  double w[32];
   double up[4][32];               // per-warp partial products (A v) over the warp's columns
   double d[TR_N], off[TR_N], o2[TR_N], gh[TR_N], y[TR_N], z[TR_N], D[TR_N], L[TR_N];
   double rd[4][8];                // per-warp results of a multiplier pass
+  double q2;                      // the secular function's derivative term at the largest left point
+  double sc[2][2];                // a step's scalars, by its parity
   int ri[4][4];
   int flag[4];
   double PL[4][TR_N][32], PR[4][TR_N][32], PY[4][TR_N][32];
 };
 
-// Newton step p = -B^-1 g by L D L^T of S.A in place, columns split over the warps.  Returns false
-// if a pivot is not positive (in every thread); otherwise lane i < 27 of every warp holds p_i.
+// Newton step p = -B^-1 g by L D L^T of S.A in place.  Returns false if a pivot is not positive (in
+// every thread); otherwise lane i < 27 of warp 0 holds p_i.
 __device__ inline bool tr_newton_step_q(TrSmemQ& S, double gi, double& p_i) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const bool row = lane < TR_N;
   double* ar = S.A + lane * TR_LD;
+  double col = row ? ar[0] : 0.0;      // warp 0: the lane's entry of column k, current
   for (int k = 0; k < TR_N; ++k) {
-    const double dk = S.A[k * TR_LD + k];
-    if (!(dk > 0.0)) return false;   // same value in every thread
-    const double r = tr_rcp(dk);
-    const bool act = row && lane > k;
-    const double li = act ? ar[k] * r : 0.0;
-    if (act) {
-      // this warp's columns j > k (j = w mod 4)
-      for (int j = k + 1 + ((w - (k + 1)) & 3); j < TR_N; j += 4) ar[j] = fma(-li, S.A[k * TR_LD + j], ar[j]);
+    const int b = k & 1, m = TR_N - 1 - k;
+    double li = 0.0;
+    if (w == 0) {
+      const double dk = __shfl_sync(0xffffffffu, col, k);
+      const double r = tr_rcp(dk);
+      if (row && lane > k) {
+        li = col * r;
+        S.v[b][lane] = li;
+        ar[k] = li;   // L below the diagonal
+      }
+      if (lane == k) {
+        S.D[k] = r;
+        S.sc[b][0] = dk;
+      }
     }
-    __syncthreads();   // row k + 1 and column k + 1 complete; every warp has read column k
-    if (act && w == (k & 3)) ar[k] = li;   // L below the diagonal (column k is not read again)
-    if (tid == k) S.D[k] = r;
+    __syncthreads();   // the step's factors; the trailing block of the previous step
+    if (!tr_positive(S.sc[b][0])) return false;
+    if (w == 0) {
+      // column k + 1, kept in registers
+      if (m > 0 && row && lane > k) col = fma(-li, S.A[k * TR_LD + k + 1], ar[k + 1]);
+    } else if (m > 1) {
+      // rows k + 1 .., columns k + 2 ..
+      const double *l = S.v[b] + k + 1, *rk = S.A + k * TR_LD + k + 2;
+      double* T = S.A + (k + 1) * TR_LD + k + 2;
+      for (TrWalk q(tid - 32, 96, m - 1); q.i < m; q.next())
+        T[q.i * TR_LD + q.j] = fma(-l[q.i], rk[q.j], T[q.i * TR_LD + q.j]);
+    }
   }
-  __syncthreads();
-  // L y = -g (column by column), y *= D^-1, L^T x = y (from the bottom); every warp alike
-  double y = row ? -gi : 0.0;
-  for (int k = 0; k < TR_N - 1; ++k) {
-    const double yk = __shfl_sync(0xffffffffu, y, k);
-    if (row && lane > k) y = fma(-ar[k], yk, y);
+  // L y = -g (column by column), y *= D^-1, L^T x = y (from the bottom)
+  if (w == 0) {
+    __syncwarp();
+    double y = row ? -gi : 0.0;
+    for (int k = 0; k < TR_N - 1; ++k) {
+      const double yk = __shfl_sync(0xffffffffu, y, k);
+      if (row && lane > k) y = fma(-ar[k], yk, y);
+    }
+    if (row) y *= S.D[lane];
+    for (int k = TR_N - 1; k > 0; --k) {
+      const double xk = __shfl_sync(0xffffffffu, y, k);
+      if (lane < k) y = fma(-S.A[k * TR_LD + lane], xk, y);
+    }
+    p_i = row ? y : 0.0;
   }
-  if (row) y *= S.D[lane];
-  for (int k = TR_N - 1; k > 0; --k) {
-    const double xk = __shfl_sync(0xffffffffu, y, k);
-    if (lane < k) y = fma(-S.A[k * TR_LD + lane], xk, y);
-  }
-  p_i = row ? y : 0.0;
   return true;
+}
+
+// The four-warp search's candidate factors (TR_FAC_Q per candidate, at fac[c + 128 q]: gfac, nfac, ufac,
+// hfac of tr_lambda_q), formed once per batch of solves.
+constexpr int TR_FAC_Q = 4;
+__device__ inline void tr_fac_q(int c, double* fac) {
+  fac[c] = c < 64 ? exp2(-0.75 * (double)(64 - c)) : (double)(c - 63) / 65.0;
+  fac[c + 128] = exp2(-0.75 * (double)((c & 63) + (c < 64 ? 0 : 1)));
+  fac[c + 256] = (double)(c - 1) / 111.0;
+  fac[c + 384] = exp2((double)(c - 64) / 8.0 + 0.0625);
 }
 
 // Copies candidate (warp src_w, lane src_l)'s y into S.y; a barrier after, so that the candidate's
@@ -90,18 +126,16 @@ __device__ inline void tr_take_y_q(TrSmemQ& S, int src_w, int src_l) {
 // point and 120-127 below the Newton point at 2^-2 .. 2^-16 of the distance to the bracket's ends.
 // Same return values as tr_lambda_parallel, in every thread.
 __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta, bool try_zero, double spec,
-                                  double hint, double& lam_out) {
+                                  double hint, const double* fac, double& lam_out) {
   constexpr double TOL = 1e-10;
+  const double rdelta = tr_rcp(delta);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, c = tid;
   double L = lo, H = hi, lamH = hi;
   bool have_h = false;
   double lamN = -1.0, lamS = -1.0;
   double lamL = -INFINITY, phiL = 0.0, dphiL = 1.0, phiH = 0.0;
-  const double gfac = c < 64 ? exp2(-0.75 * (double)(64 - c)) : (double)(c - 63) / 65.0;
-  const double nfac = exp2(-0.75 * (double)((c & 63) + (c < 64 ? 0 : 1)));
-  const double ufac = (double)(c - 1) / 111.0;
-  const double afac = exp2(-2.0 * (double)((c & 7) + 1));
-  const double hfac = exp2((double)(c - 64) / 8.0 + 0.0625);
+  const double gfac = fac[c], nfac = fac[c + 128], ufac = fac[c + 256], hfac = fac[c + 384];
+  const double afac = tr_pow2(-2 * ((c & 7) + 1));
   for (int pass = 0; pass < 16; ++pass) {
     double lam;
     const double span = H - L;
@@ -120,8 +154,8 @@ __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta
       if (lh > L && lh < H) lam = lh;
     }
     __syncwarp();
-    double pn = 0.0, qn2 = 0.0;
-    const bool pd = tr_eval_lane(S, S.PL[w], S.PR[w], S.PY[w], lane, lam, pn, qn2);
+    double pn = 0.0;
+    const bool pd = tr_eval_lane(S, S.PL[w], S.PR[w], S.PY[w], lane, lam, pn);
     // ---- this warp's part: best error, bracket ends, largest left point
     const double err = pd ? fabs(pn - delta) : INFINITY;
     const double bw = tr_warp_min(err);
@@ -136,7 +170,7 @@ __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta
     const double lbw = tr_warp_max(lft ? lam : -INFINITY);
     const unsigned ml = __ballot_sync(0xffffffffu, lft && lam == lbw);
     const int ilw = ml ? __ffs(ml) - 1 : 0;
-    const double pnbw = __shfl_sync(0xffffffffu, pn, ilw), qbw = __shfl_sync(0xffffffffu, qn2, ilw);
+    const double pnbw = __shfl_sync(0xffffffffu, pn, ilw);
     const double lamBw = __shfl_sync(0xffffffffu, lam, iw);
     const int int0 = __shfl_sync(0xffffffffu, (int)(pd && pn <= delta), 0);
     if (lane == 0) {
@@ -146,8 +180,7 @@ __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta
       S.rd[w][3] = pnHw;
       S.rd[w][4] = lbw;
       S.rd[w][5] = pnbw;
-      S.rd[w][6] = qbw;
-      S.rd[w][7] = lamBw;
+      S.rd[w][6] = lamBw;
       S.ri[w][0] = iw;
       S.ri[w][1] = iHw;
       S.ri[w][2] = int0;
@@ -163,7 +196,7 @@ __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta
     for (int q = 1; q < 4; ++q)
       if (S.rd[q][0] < S.rd[wb][0]) wb = q;
     if (S.rd[wb][0] <= TOL * delta) {
-      lam_out = S.rd[wb][7];
+      lam_out = S.rd[wb][6];
       tr_take_y_q(S, wb, S.ri[wb][0]);
       return 0;
     }
@@ -175,23 +208,26 @@ __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta
       if (S.rd[q][4] > S.rd[wl][4]) wl = q;
     }
     const double newH = S.rd[wh][2], pnH = S.rd[wh][3];
-    const double lbest = S.rd[wl][4], pnb = S.rd[wl][5], qb = S.rd[wl][6];
+    const double lbest = S.rd[wl][4], pnb = S.rd[wl][5];
     const int iH = S.ri[wh][1];
-    // every thread has read rd / ri; the copy's barrier orders them before the next pass's writes
+    const bool more_l = lbest > lamL;
+    if (newH < H && tid < TR_N) S.y[tid] = S.PY[wh][tid][iH];
+    if (more_l && w == wl) {
+      const double q2 = tr_q2_lane(S.PL[w], S.PR[w], S.PY[w], lane);
+      if (lane == ilw) S.q2 = q2;
+    }
+    __syncthreads();   // y and q2 published; rd, ri and the warps' scratch read before the next pass's writes
     if (newH < H) {
-      tr_take_y_q(S, wh, iH);
       H = newH;
       lamH = newH;
-      phiH = tr_rcp(pnH) - tr_rcp(delta);
+      phiH = tr_rcp(pnH) - rdelta;
       have_h = true;
-    } else {
-      __syncthreads();
     }
     L = fmax(L, newL);
-    if (lbest > lamL) {
+    if (more_l) {
       lamL = lbest;
-      phiL = tr_rcp(pnb) - tr_rcp(delta);
-      dphiL = qb * tr_rcp(pnb * pnb * pnb);
+      phiL = tr_rcp(pnb) - rdelta;
+      dphiL = S.q2 * tr_rcp(pnb * pnb * pnb);
     }
     lamN = lamL > -INFINITY ? lamL - phiL * tr_rcp(dphiL) : -1.0;
     lamS = have_h && lamL > -INFINITY && phiH > phiL ? lamL + (H - lamL) * (-phiL * tr_rcp(phiH - phiL)) : -1.0;
@@ -210,7 +246,8 @@ __device__ inline int tr_lambda_q(TrSmemQ& S, double lo, double hi, double delta
 // and warp 0 holds pred, hard and lam_out (every warp, when the Newton step was taken).
 __device__ inline bool tr_solve_q(TrSmemQ& S, const double* __restrict__ Bsrc, double bsign, double gi, double delta,
                                   bool try_newton, const double* __restrict__ cache_in, double* __restrict__ cache_out,
-                                  double lam_hint, double& lam_out, double& p_i, double& pred, int& hard) {
+                                  double lam_hint, const double* fac, double& lam_out, double& p_i, double& pred,
+                                  int& hard) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int n = TR_N;
   const bool row = lane < n;
@@ -230,14 +267,20 @@ __device__ inline bool tr_solve_q(TrSmemQ& S, const double* __restrict__ Bsrc, d
     if (try_newton) {
       for (int i = tid; i < TR_N * TR_N; i += 128) S.A[i] = bsign * Bsrc[i];
       __syncthreads();
-      double pn;
+      double pn = 0.0;
       const bool pdef = tr_newton_step_q(S, gi, pn);
       if (pdef) {
-        const double pp = tr_warp_sum(pn * pn);
-        if (sqrt(pp) <= delta) {
-          p_i = pn;
-          pred = -0.5 * tr_warp_sum(gi * pn);
-          hard = 0;
+        if (w == 0) {
+          const double pp = tr_warp_sum(pn * pn);
+          if (lane == 0) S.flag[3] = sqrt(pp) <= delta;
+        }
+        __syncthreads();
+        if (S.flag[3]) {
+          if (w == 0) {
+            p_i = pn;
+            pred = -0.5 * tr_warp_sum(gi * pn);
+            hard = 0;
+          }
           lam_out = 0.0;
           return false;
         }
@@ -246,67 +289,94 @@ __device__ inline bool tr_solve_q(TrSmemQ& S, const double* __restrict__ Bsrc, d
     }
     for (int i = tid; i < TR_N * TR_N; i += 128) S.A[i] = bsign * Bsrc[i];
     __syncthreads();
-    // ---- Householder tridiagonalisation: lane i owns row i, warp w the columns j = w mod 4
+    // ---- Householder tridiagonalisation.  Step k: warp 0 (lane i: row i) holds column k, current, in
+    //      `col`; it forms the reflection and publishes it; every warp multiplies its columns; warp 0
+    //      forms w and, from it, column k + 1, warp 1 reflects g (lane i holds gh_i); warps 1-3 then
+    //      update rows and columns k + 2 .. while warp 0 goes on with column k + 1.
     double gh = row ? gi : 0.0;
     double* ar = S.A + lane * TR_LD;
+    double col = row ? ar[0] : 0.0;
     for (int k = 0; k < n - 2; ++k) {
-      const double xi = lane > k && row ? ar[k] : 0.0;
-      const double s2 = tr_warp_sum(xi * xi);
-      const double x0 = S.A[(k + 1) * TR_LD + k];
-      if (s2 == 0.0) {   // same in every warp
-        if (tid == 0) {
-          S.beta[k] = 0.0;
-          S.off[k + 1] = 0.0;
+      const int b = k & 1, m = n - 1 - k;
+      double vi = 0.0;
+      if (w == 0) {
+        if (lane == k) S.d[k] = col;   // the diagonal entry is final
+        const double xi = lane > k && row ? col : 0.0;
+        const double s2 = tr_warp_sum(xi * xi);
+        const double x0 = __shfl_sync(0xffffffffu, col, k + 1);
+        double alpha = 0.0, beta = 0.0;
+        if (s2 != 0.0) {   // same in every lane
+          alpha = -copysign(sqrt(s2), x0);
+          vi = lane == k + 1 ? x0 - alpha : xi;
+          beta = tr_rcp(s2 - alpha * x0);   // 2 / v.v with v.v = 2 (s2 - alpha x0)
+          S.v[b][lane] = vi;
+          if (lane > k && row) ar[k] = vi;   // keep the reflection vector
+        }
+        if (lane == 0) {
+          S.sc[b][0] = s2;
+          S.sc[b][1] = beta;
+          S.beta[k] = beta;
+          S.off[k + 1] = alpha;
+        }
+      }
+      __syncthreads();   // (a) the reflection; the previous step's update
+      if (S.sc[b][0] == 0.0) {   // same in every thread: nothing to reflect
+        if (w == 0 && row && lane > k) {
+          ar[k] = col;
+          col = ar[k + 1];
         }
         continue;
       }
-      const double alpha = -copysign(sqrt(s2), x0);
-      const double vi = lane == k + 1 ? x0 - alpha : xi;
-      const double beta = tr_rcp(s2 - alpha * x0);
-      S.v[w][lane] = vi;
-      __syncwarp();
+      const double beta = S.sc[b][1];
       const int j0 = k + 1 + ((w - (k + 1)) & 3);   // this warp's first column > k
       double u0 = 0.0, u1 = 0.0;
       if (lane > k && row) {
         int j = j0;
         for (; j + 4 < n; j += 8) {
-          u0 = fma(ar[j], S.v[w][j], u0);
-          u1 = fma(ar[j + 4], S.v[w][j + 4], u1);
+          u0 = fma(ar[j], S.v[b][j], u0);
+          u1 = fma(ar[j + 4], S.v[b][j + 4], u1);
         }
-        if (j < n) u0 = fma(ar[j], S.v[w][j], u0);
+        if (j < n) u0 = fma(ar[j], S.v[b][j], u0);
       }
       S.up[w][lane] = u0 + u1;
-      __syncthreads();   // (a) the four partial products
-      const double u = (S.up[0][lane] + S.up[1][lane]) + (S.up[2][lane] + S.up[3][lane]);
-      const double pi = beta * u;
-      double vp = vi * pi, vg = vi * gh;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        vp += __shfl_xor_sync(0xffffffffu, vp, o);
-        vg += __shfl_xor_sync(0xffffffffu, vg, o);
+      __syncthreads();   // (b) the four partial products
+      if (w == 0) {
+        const double u = (S.up[0][lane] + S.up[1][lane]) + (S.up[2][lane] + S.up[3][lane]);
+        const double pi = beta * u;
+        const double vp = tr_warp_sum(vi * pi);
+        const double K = 0.5 * beta * vp;
+        const double wi = pi - K * vi;
+        S.w[lane] = wi;
+        // column k + 1
+        const double w1 = __shfl_sync(0xffffffffu, wi, k + 1), v1 = __shfl_sync(0xffffffffu, vi, k + 1);
+        if (lane > k && row) col = fma(-vi, w1, fma(-wi, v1, ar[k + 1]));
+      } else if (w == 1) {
+        vi = S.v[b][lane];
+        const double vg = tr_warp_sum(vi * gh);
+        gh = fma(-beta * vg, vi, gh);
       }
-      const double K = 0.5 * beta * vp;
-      const double wi = pi - K * vi;
-      gh = fma(-beta * vg, vi, gh);
-      S.w[w][lane] = wi;
-      __syncwarp();
-      if (lane > k && row) {
-        for (int j = j0; j < n; j += 4) ar[j] = fma(-vi, S.w[w][j], fma(-wi, S.v[w][j], ar[j]));
-        if (w == (k & 3)) ar[k] = vi;   // the reflection vector (column k is not read again)
+      __syncthreads();   // (c) w
+      if (w > 0 && m > 1) {
+        const double *v = S.v[b] + k + 2, *ww = S.w + k + 2;
+        double* T = S.A + (k + 2) * TR_LD + k + 2;
+        for (TrWalk q(tid - 32, 96, m - 1); q.i < m - 1; q.next()) {
+          double* t = T + q.i * TR_LD + q.j;
+          *t = fma(-v[q.i], ww[q.j], fma(-ww[q.i], v[q.j], *t));
+        }
       }
-      if (tid == 0) {
-        S.beta[k] = beta;
-        S.off[k + 1] = alpha;
-      }
-      __syncthreads();   // (b) column k + 1 complete before the next step reads it
     }
-    if (tid < n) S.d[tid] = S.A[tid * TR_LD + tid];
-    if (w == 0 && row) S.gh[lane] = gh;
-    if (tid == 0) {
-      S.off[n - 1] = S.A[(n - 1) * TR_LD + n - 2];
-      S.off[0] = 0.0;
+    // the last 2 x 2 block: its first column is in warp 0's registers
+    if (w == 0) {
+      if (lane == n - 2) S.d[n - 2] = col;
+      if (lane == n - 1) S.off[n - 1] = col;
+      if (lane == 0) S.off[0] = 0.0;
+      // (the stored block keeps column n - 2 as the one-warp solver leaves it)
+      if (lane >= n - 2 && row) ar[n - 2] = col;
+    } else if (w == 1 && row) {
+      S.gh[lane] = gh;
     }
     __syncthreads();
+    if (tid == 0) S.d[n - 1] = S.A[(n - 1) * TR_LD + n - 1];
     if (tid < n) S.o2[tid] = S.off[tid] * S.off[tid];
     __syncthreads();
     if (cache_out) {
@@ -336,7 +406,7 @@ __device__ inline bool tr_solve_q(TrSmemQ& S, const double* __restrict__ Bsrc, d
   if (tid == 0) S.flag[2] = 0;
   __syncthreads();
   lam_out = -1.0;
-  const int hc = tr_lambda_q(S, lo, hi, delta, lo == 0.0, spec, lam_hint, lam_out);
+  const int hc = tr_lambda_q(S, lo, hi, delta, lo == 0.0, spec, lam_hint, fac, lam_out);
   if (hc) {
     lam_out = -1.0;
     // hard case on warp 0, as in tr_solve_warp
