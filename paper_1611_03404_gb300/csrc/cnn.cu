@@ -478,27 +478,23 @@ extern "C" int celeste_cnn_forward_ex(const float* params, const uint16_t* param
     int* err = nullptr;
     if ((e = cudaGetSymbolAddress(reinterpret_cast<void**>(&err), g_cnn_tc_err)) != cudaSuccess)
       return cuda_fail(e, "cnn error word");
-    auto conv = [&](const ConvGeom& g, const bf16* in, int64_t wo, int64_t bo, bf16* out) {
+    int dev = 0, n_sm = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return cuda_fail(e, "SM count");
+    auto layer = [&](cnn_tc::LayerId id, int m, int n, const bf16* in, int64_t wo, int64_t bo, bf16* out, float* outf) {
       cnn_tc::Args a{};
-      a.M = g.B * g.OH * g.OW;
-      a.N = g.Cout;
-      a.K = 9 * g.Cin;
-      a.conv = 1;
-      a.B = g.B, a.H = g.H, a.W = g.W, a.Cin = g.Cin, a.OH = g.OH, a.OW = g.OW, a.stride = g.stride;
-      a.in = in, a.w = pb + wo, a.bias = params + bo, a.out = out, a.err = err;
-      return tc_gemm_forward(a, st);
+      a.M = m, a.N = n, a.B = B;
+      a.in = in, a.w = pb + wo, a.bias = params + bo, a.out = out, a.out_f = outf, a.err = err;
+      if (outf) a.scale = out_scale, a.shift = out_shift;
+      return tc_forward(id, a, n_sm, st);
     };
-    auto fc = [&](int nin, int nout, const bf16* in, int64_t wo, int64_t bo, bf16* out, float* outf) {
-      cnn_tc::Args a{};
-      a.M = B, a.N = nout, a.K = nin, a.conv = 0;
-      a.in = in, a.w = pb + wo, a.bias = params + bo, a.out = out, a.out_f = outf, a.scale = out_scale,
-      a.shift = out_shift, a.err = err;
-      return tc_gemm_forward(a, st);
-    };
-    if ((e = conv(g1, xin, o.w1, o.b1, w.a1)) != cudaSuccess || (e = conv(g2, w.a1, o.w2, o.b2, w.a2)) != cudaSuccess ||
-        (e = conv(g3, w.a2, o.w3, o.b3, w.a3)) != cudaSuccess || (e = conv(g4, w.a3, o.w4, o.b4, w.a4)) != cudaSuccess ||
-        (e = fc(FLAT, F5, w.a4, o.w5, o.b5, w.a5, nullptr)) != cudaSuccess ||
-        (e = fc(F5, NOUT, w.a5, o.w6, o.b6, nullptr, y)) != cudaSuccess)
+    if ((e = layer(cnn_tc::CONV1, B * 1024, C1, xin, o.w1, o.b1, w.a1, nullptr)) != cudaSuccess ||
+        (e = layer(cnn_tc::CONV2, B * 256, C2, w.a1, o.w2, o.b2, w.a2, nullptr)) != cudaSuccess ||
+        (e = layer(cnn_tc::CONV3, B * 64, C3, w.a2, o.w3, o.b3, w.a3, nullptr)) != cudaSuccess ||
+        (e = layer(cnn_tc::CONV4, B * 16, C4, w.a3, o.w4, o.b4, w.a4, nullptr)) != cudaSuccess ||
+        (e = layer(cnn_tc::DENSE1, B, F5, w.a4, o.w5, o.b5, w.a5, nullptr)) != cudaSuccess ||
+        (e = layer(cnn_tc::DENSE2, B, NOUT, w.a5, o.w6, o.b6, nullptr, y)) != cudaSuccess)
       return cuda_fail(e, "cnn forward (tensor cores)");
     return CELESTE_OK;
   }

@@ -9,12 +9,12 @@ namespace celeste {
 namespace cnn_tc {
 
 // D[M x N] = A[M x K] B[K x N]: A the layer input (im2col of a 3x3, padding-1 convolution over an
-// NHWC tensor when conv is set), B the weights [N][K] (K-major), bias [N]; D stored as BF16 after
-// ReLU into out [M][N], or as FP32 into out_f [M][N] (times scale plus shift when scale is set).
+// NHWC tensor, or [M][K]), B the weights [N][K] (K-major), bias [N]; D stored as BF16 after ReLU into
+// out [M][N], or as FP32 into out_f [M][N] (times scale plus shift when scale is set).  The kernels are
+// built for the network's layers.
+enum LayerId { CONV1, CONV2, CONV3, CONV4, DENSE1, DENSE2 };
 struct Args {
-  int M, N, K;
-  int conv;
-  int B, H, W, Cin, OH, OW, stride;
+  int M, N, B;                   // rows and columns of D, patches
   const __nv_bfloat16* in;
   const __nv_bfloat16* w;
   const float* bias;
@@ -27,6 +27,7 @@ struct Args {
 
 }  // namespace cnn_tc
 
-cudaError_t tc_gemm_forward(const cnn_tc::Args& a, cudaStream_t st);
+// n_sm: SMs of the current device.
+cudaError_t tc_forward(cnn_tc::LayerId layer, const cnn_tc::Args& a, int n_sm, cudaStream_t st);
 
 }  // namespace celeste
