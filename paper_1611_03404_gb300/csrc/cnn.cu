@@ -10,10 +10,9 @@
 //   W1 [32][3][3][5], b1 [32], W2 [64][3][3][32], b2, W3 [64][3][3][64], b3, W4 [64][3][3][64],
 //   b4, W5 [256][1024], b5 [256], W6 [27][256], b6 [27].
 //
-// Every convolution and product runs through one implicit-GEMM kernel: 64 x 64 output tiles,
-// k-steps of 32, four warps of 32 x 32 issuing mma.sync m16n8k16 (BF16 in, FP32 accumulate).
-// The operand loaders gather straight from the NHWC tensors (im2col on the fly), so forward,
-// input-gradient and weight-gradient passes differ only in their gather and epilogue.
+// The forward layers run on tcgen05 (cnn_tc.cu); the mma.sync engine kept beside them is one
+// implicit-GEMM kernel (64 x 64 output tiles, k-steps of 32, four warps of 32 x 32 on mma.sync m16n8k16,
+// operands gathered element by element).  The backward pass has its own GEMM below.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -195,51 +194,6 @@ struct ConvFwd {
   }
 };
 
-// din[b, ih, iw, ci] = [in > 0] sum_{co, kh, kw} dout[b, oh, ow, co] W[co, kh, kw, ci],
-// ih = oh s + kh - 1 (the mask turns the gradient w.r.t. the input activation into the gradient
-// w.r.t. the previous layer's pre-ReLU value)
-struct ConvDgrad {
-  ConvGeom g;
-  const bf16* dout;
-  const bf16* w;
-  const bf16* in;
-  bf16* din;
-  __device__ bf16 a(int m, int k) const {
-    const int iw = m % g.W, r = m / g.W, ih = r % g.H, b = r / g.H;
-    const int co = k % g.Cout, kk = k / g.Cout, kh = kk / 3, kw = kk % 3;
-    const int th = ih + 1 - kh, tw = iw + 1 - kw;
-    if (th < 0 || tw < 0 || th % g.stride || tw % g.stride) return bzero();
-    const int oh = th / g.stride, ow = tw / g.stride;
-    if (oh >= g.OH || ow >= g.OW) return bzero();
-    return dout[(((size_t)b * g.OH + oh) * g.OW + ow) * g.Cout + co];
-  }
-  __device__ bf16 b(int k, int n) const {
-    const int co = k % g.Cout, kk = k / g.Cout;
-    return w[((size_t)co * 9 + kk) * g.Cin + n];
-  }
-  __device__ void store(int m, int n, float v) const {
-    const size_t i = (size_t)m * g.Cin + n;
-    din[i] = __float2bfloat16(__bfloat162float(in[i]) > 0.f ? v : 0.f);
-  }
-};
-
-// dW[co, kh, kw, ci] += sum_{b, oh, ow} dout[b, oh, ow, co] in[b, oh s + kh - 1, ow s + kw - 1, ci]
-struct ConvWgrad {
-  ConvGeom g;
-  const bf16* dout;
-  const bf16* in;
-  float* dw;
-  __device__ bf16 a(int m, int k) const { return dout[(size_t)k * g.Cout + m]; }
-  __device__ bf16 b(int k, int n) const {
-    const int ow = k % g.OW, r = k / g.OW, oh = r % g.OH, b = r / g.OH;
-    const int ci = n % g.Cin, kk = n / g.Cin, kh = kk / 3, kw = kk % 3;
-    const int ih = oh * g.stride + kh - 1, iw = ow * g.stride + kw - 1;
-    if (ih < 0 || ih >= g.H || iw < 0 || iw >= g.W) return bzero();
-    return in[(((size_t)b * g.H + ih) * g.W + iw) * g.Cin + ci];
-  }
-  __device__ void store(int m, int n, float v) const { atomicAdd(dw + (size_t)m * 9 * g.Cin + n, v); }
-};
-
 // ------------------------------------------------------------------------------ dense ops
 // y[b, o] = act(bias[o] + sum_i x[b, i] W[o, i]); the last layer writes FP32, optionally mapped
 // to parameter space as y * scale[o] + shift[o].
@@ -265,51 +219,479 @@ struct FcFwd {
   }
 };
 
-// dx[b, i] = [x > 0] sum_o dy[b, o] W[o, i]   (dy BF16, or FP32 for the last layer)
-template <class T>
-struct FcDgrad {
-  int Nin, Nout;
-  const T* dy;
-  const bf16* w;
-  const bf16* x;
-  bf16* dx;
-  __device__ bf16 a(int m, int k) const { return __float2bfloat16((float)dy[(size_t)m * Nout + k]); }
-  __device__ bf16 b(int k, int n) const { return w[(size_t)k * Nin + n]; }
-  __device__ void store(int m, int n, float v) const {
-    const size_t i = (size_t)m * Nin + n;
-    dx[i] = __float2bfloat16(__bfloat162float(x[i]) > 0.f ? v : 0.f);
+// ------------------------------------------------------------------------------ backward GEMM
+// C[M x N] = sum_k A(m, k) B(k, n) on mma.sync m16n8k16 (BF16 in, FP32 accumulate), operands brought in
+// 16-byte chunks by cp.async, three stages of 64 x 64 deep, read with ldmatrix.  A lies in memory either
+// with k contiguous (rows m: the input gradients) or with m contiguous (rows k: the weight gradients), B
+// always with n contiguous (rows k); ldmatrix.trans turns the latter two.  blockIdx.z splits K, or is the
+// operation's own index (parity classes of an input gradient).
+// What bounds it: reading the operands (a layer's gradients from L2 at the training batch); before, every
+// element was gathered and converted on its own, and an input gradient multiplied the three quarters of
+// a stride-2 layer's taps that are zero.  A whole training step at batch 512:
+// 4.75 ms before, 0.31 now, of which 0.21 is the backward pass.
+constexpr int BK2 = 64, LD2 = 72, STAGES2 = 3;     // rows of 64 values, 16 bytes apart from a multiple of 128
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// 16 bytes global -> shared, asynchronously; zeros where !ok (the source is then not read).
+__device__ __forceinline__ void copy16(void* dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+// The same from a caller's array, which may start off a 16-byte boundary (then element by element, visible
+// after the next barrier).
+__device__ __forceinline__ void copy16_any(bf16* dst, const bf16* src, bool ok) {
+  if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    copy16(dst, src, ok);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) dst[i] = ok ? src[i] : __float2bfloat16(0.f);
+  }
+}
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
+}
+
+// A 16 x 16 operand block at (row, col) of a tile with rows of LD values: as A from [m][k], as A from
+// [k][m], and as two adjacent B blocks (n .. n + 15) from [k][n].
+template <int LD>
+__device__ __forceinline__ void frag_a(uint32_t (&r)[4], const bf16* T, int m, int k, int lane) {
+  ldsm4(r, T + (m + (lane & 15)) * LD + k + 8 * (lane >> 4));
+}
+template <int LD>
+__device__ __forceinline__ void frag_at(uint32_t (&r)[4], const bf16* T, int m, int k, int lane) {
+  ldsm4t(r, T + (k + (lane & 7) + 8 * (lane >> 4)) * LD + m + 8 * ((lane >> 3) & 1));
+}
+template <int LD>
+__device__ __forceinline__ void frag_b(uint32_t (&r)[4], const bf16* T, int k, int n, int lane) {
+  ldsm4t(r, T + (k + (lane & 15)) * LD + n + 8 * (lane >> 4));
+}
+
+template <class Op>
+__global__ void __launch_bounds__(128) bwd_gemm_kernel(Op op, int M, int N, int K, int k_chunk) {
+  constexpr int BN2 = Op::BN;                       // 64, or 32 (then a warp takes 16 rows of C, else 32)
+  constexpr int MI = BN2 == 64 ? 2 : 1;             // 16-row blocks per warp; always 32 columns
+  extern __shared__ __align__(16) unsigned char dyn[];
+  bf16* const As = reinterpret_cast<bf16*>(dyn);
+  bf16* const Bs = As + STAGES2 * 64 * LD2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int m0 = blockIdx.x * 64, n0 = blockIdx.y * BN2;
+  const int wm = MI == 2 ? (warp >> 1) * 32 : warp * 16, wn = MI == 2 ? (warp & 1) * 32 : 0;
+  const int c = tid & 7, r0 = tid >> 3;             // this thread's chunk and first row (then every 16th)
+  int kb, ke;
+  op.range(blockIdx.z, k_chunk, K, kb, ke);
+  op.rows(m0, r0, M);                               // what the thread's rows need for all of K
+  const int steps = (ke - kb + BK2 - 1) / BK2;
+  auto fetch = [&](int s) {
+    if (s < steps) {
+      const int k0 = kb + s * BK2;
+      bf16* A = As + (s % STAGES2) * 64 * LD2;
+      bf16* B = Bs + (s % STAGES2) * 64 * LD2;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = r0 + 16 * i;
+        bool ok;
+        const bf16* p = Op::A_K ? op.a(i, k0, k0 + 8 * c, ke, ok) : op.at(k0 + r, m0 + 8 * c, M, ke, ok);
+        copy16(A + r * LD2 + 8 * c, ok ? p : op.any(), ok);
+        if (8 * c < BN2) {
+          const bf16* q = op.b(k0, k0 + r, n0 + 8 * c, N, ke, ok);
+          copy16_any(B + r * LD2 + 8 * c, ok ? q : op.any(), ok);
+        }
+      }
+    }
+    cp_async_commit();
+  };
+  float acc[MI][4][4];
+#pragma unroll
+  for (int i = 0; i < MI; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+  fetch(0);
+  fetch(1);
+  for (int s = 0; s < steps; ++s) {
+    copy_wait<1>();
+    __syncthreads();   // step s is there for every thread; step s - 1 has been read
+    fetch(s + 2);
+    const bf16* A = As + (s % STAGES2) * 64 * LD2;
+    const bf16* B = Bs + (s % STAGES2) * 64 * LD2;
+#pragma unroll
+    for (int kk = 0; kk < BK2; kk += 16) {
+      if (kb + s * BK2 + kk >= ke) break;            // (blocks past K hold zeros)
+      uint32_t a[MI][4], b[2][4];
+#pragma unroll
+      for (int i = 0; i < MI; ++i) {
+        if constexpr (Op::A_K) frag_a<LD2>(a[i], A, wm + 16 * i, kk, lane);
+        else frag_at<LD2>(a[i], A, wm + 16 * i, kk, lane);
+      }
+#pragma unroll
+      for (int j = 0; j < 2; ++j) frag_b<LD2>(b[j], B, kk, wn + 16 * j, lane);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < MI; ++i) mma16816(acc[i][j], a[i], b[j >> 1][2 * (j & 1)], b[j >> 1][2 * (j & 1) + 1]);
+    }
+  }
+  copy_wait<0>();
+  const int g = lane >> 2, t = lane & 3;
+  if constexpr (Op::SUM) {
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int m = m0 + wm + 16 * i + g + (e >> 1) * 8, n = n0 + wn + 8 * j + 2 * t + (e & 1);
+          if (m < M && n < N) op.add(m, n, acc[i][j][e]);
+        }
+  } else {
+    // BF16 rows of the tile through shared memory, then 16 bytes of a row per thread
+    __syncthreads();
+    bf16* C = As;
+#pragma unroll
+    for (int i = 0; i < MI; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<__nv_bfloat162*>(C + (wm + 16 * i + g + 8 * h) * LD2 + wn + 8 * j + 2 * t) =
+              __floats2bfloat162_rn(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+    __syncthreads();
+    for (int e = tid; e < 64 * (BN2 / 8); e += 128) {
+      const int r = e / (BN2 / 8), ch = e % (BN2 / 8), m = m0 + r, n = n0 + 8 * ch;
+      if (m < M && n < N) op.store(blockIdx.z, m, n, *reinterpret_cast<const uint4*>(C + r * LD2 + 8 * ch));
+    }
+  }
+}
+
+template <class Op>
+cudaError_t bwd_gemm(const Op& op, int M, int N, int K, int z, int k_chunk, cudaStream_t st) {
+  constexpr int smem = 2 * STAGES2 * 64 * LD2 * (int)sizeof(bf16);
+  cudaError_t e = cudaFuncSetAttribute(bwd_gemm_kernel<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  bwd_gemm_kernel<Op><<<dim3((M + 63) / 64, (N + Op::BN - 1) / Op::BN, z), 128, smem, st>>>(op, M, N, K, k_chunk);
+  return cudaGetLastError();
+}
+
+// The value where the layer's activation was positive, else 0 (the gradient w.r.t. the pre-ReLU value).
+__device__ __forceinline__ uint4 relu_mask(uint4 v, const bf16* act) {
+  const uint4 x = *reinterpret_cast<const uint4*>(act);
+  auto one = [](uint32_t v, uint32_t x) {
+    // positive BF16: sign clear, not zero (activations are never NaN after ReLU's maximum)
+    const uint32_t lo = (x & 0x8000u) == 0 && (x & 0x7fffu) ? 0xffffu : 0u;
+    const uint32_t hi = (x & 0x80000000u) == 0 && (x & 0x7fff0000u) ? 0xffff0000u : 0u;
+    return v & (lo | hi);
+  };
+  return make_uint4(one(v.x, x.x), one(v.y, x.y), one(v.z, x.z), one(v.w, x.w));
+}
+
+// Input gradient of a 3x3, stride-2, padding-1 convolution with 64 output channels, one parity class of the
+// input pixels (z = 2 (ih & 1) + (iw & 1)) at a time: an even coordinate is reached by tap 1 alone, an odd one by
+// taps 0 (from the next output) and 2, so the classes have 1, 2, 2 and 4 taps, taken in ascending order.
+// Rows: (b, ih / 2, iw / 2).  din = [in > 0] sum_{taps, co} dout[b, oh, ow, co] W[co, kh, kw, ci].
+template <int O, int CIN>
+struct ConvDgrad {
+  static constexpr bool A_K = true, SUM = false;
+  static constexpr int BN = CIN;
+  const bf16 *dout, *w, *in;
+  bf16* din;
+  int pi, pj;
+  const bf16* row[4];
+  int edge[4];   // 1: no output below, 2: none to the right, 4: no row at all
+  __device__ const bf16* any() const { return w; }
+  __device__ void range(int z, int, int, int& kb, int& ke) {
+    pi = z >> 1;
+    pj = z & 1;
+    kb = 0;
+    ke = 64 * (1 + pi) * (1 + pj);
+  }
+  __device__ void rows(int m0, int r0, int M) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = m0 + r0 + 16 * i, j = m % O, y = m / O % O;
+      row[i] = dout + (int64_t)m * 64;
+      edge[i] = (y == O - 1 ? 1 : 0) | (j == O - 1 ? 2 : 0) | (m >= M ? 4 : 0);
+    }
+  }
+  // tap number t of the class: output offsets (dh, dw), kernel position
+  __device__ void tap(int t, int& dh, int& dw, int& kk) const {
+    const int th = pj ? t >> 1 : t, tw = pj ? t & 1 : 0;
+    dh = pi ? 1 - th : 0;
+    dw = pj ? 1 - tw : 0;
+    kk = 3 * (pi ? 2 * th : 1) + (pj ? 2 * tw : 1);
+  }
+  __device__ const bf16* a(int i, int k0, int k, int, bool& ok) const {
+    int dh, dw, kk;
+    tap(k0 >> 6, dh, dw, kk);
+    ok = !(edge[i] & (4 | dh | (dw << 1)));
+    return row[i] + (dh * O + dw) * 64 + (k & 63);
+  }
+  __device__ const bf16* at(int, int, int, int, bool&) const { return nullptr; }
+  __device__ const bf16* b(int k0, int k, int n, int, int, bool& ok) const {
+    int dh, dw, kk;
+    tap(k0 >> 6, dh, dw, kk);
+    ok = true;
+    return w + ((k & 63) * 9 + kk) * CIN + n;
+  }
+  __device__ void store(int z, int m, int n, uint4 v) const {
+    const int j = m % O, y = m / O % O, b = m / (O * O);
+    const int64_t at = (((int64_t)b * (2 * O) + 2 * y + (z >> 1)) * (2 * O) + 2 * j + (z & 1)) * CIN + n;
+    *reinterpret_cast<uint4*>(din + at) = relu_mask(v, in + at);
+  }
+  __device__ void add(int, int, float) const {}
+};
+
+// K split of the weight gradients.
+struct SplitK {
+  __device__ static void range(int z, int chunk, int K, int& kb, int& ke) {
+    kb = z * chunk;
+    ke = min(K, kb + chunk);
   }
 };
 
-// dW[o, i] += sum_b dy[b, o] x[b, i]
-template <class T>
-struct FcWgrad {
-  int Nin, Nout;
-  const T* dy;
-  const bf16* x;
+// Weight gradient of the same convolutions: dW[co, tap, ci] += sum_px dout[px, co] in[px's tap, ci].
+template <int O, int CIN>
+struct ConvWgrad : SplitK {
+  static constexpr bool A_K = false, SUM = true;
+  static constexpr int BN = 64;
+  const bf16 *dout, *in;
   float* dw;
-  __device__ bf16 a(int m, int k) const { return __float2bfloat16((float)dy[(size_t)k * Nout + m]); }
-  __device__ bf16 b(int k, int n) const { return x[(size_t)k * Nin + n]; }
-  __device__ void store(int m, int n, float v) const { atomicAdd(dw + (size_t)m * Nin + n, v); }
+  __device__ const bf16* any() const { return in; }
+  __device__ void rows(int, int, int) {}
+  __device__ const bf16* a(int, int, int, int, bool&) const { return nullptr; }
+  __device__ const bf16* at(int k, int m, int, int ke, bool& ok) const {
+    ok = k < ke;
+    return dout + (int64_t)k * 64 + m;
+  }
+  __device__ const bf16* b(int, int k, int n, int N, int ke, bool& ok) const {
+    const int tap = n / CIN, kh = tap / 3, kw = tap % 3, ow = k % O, oh = k / O % O, b = k / (O * O);
+    const int y = 2 * oh + kh - 1, x = 2 * ow + kw - 1;   // (never past the lower or right edge)
+    ok = k < ke && n < N && y >= 0 && x >= 0;
+    return in + (((int64_t)b * (2 * O) + y) * (2 * O) + x) * CIN + n % CIN;
+  }
+  __device__ void add(int m, int n, float v) const { atomicAdd(dw + m * 9 * CIN + n, v); }
+  __device__ void store(int, int, int, uint4) const {}
 };
 
-// db[c] += sum over rows of g[r, c]
-template <class T>
-__global__ void bias_grad_kernel(const T* g, int64_t rows, int C, float* db) {
-  const int c = threadIdx.x % C, lanes = blockDim.x / C;
-  if ((int)threadIdx.x >= lanes * C) return;
-  float s = 0.f;
-  for (int64_t r = (int64_t)blockIdx.x * lanes + threadIdx.x / C; r < rows; r += (int64_t)gridDim.x * lanes)
-    s += (float)g[r * C + c];
-  atomicAdd(db + c, s);
+// Dense layers; dy [B][LDY] with NOUT values in use.
+// dx[b, i] = [x > 0] sum_o dy[b, o] W[o, i]
+template <int NIN, int NOUT, int LDY>
+struct FcDgrad : SplitK {
+  static constexpr bool A_K = true, SUM = false;
+  static constexpr int BN = 64;
+  const bf16 *dy, *w, *x;
+  bf16* dx;
+  const bf16* row[4];
+  bool in_range[4];
+  __device__ const bf16* any() const { return w; }
+  __device__ void rows(int m0, int r0, int M) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      row[i] = dy + (int64_t)(m0 + r0 + 16 * i) * LDY;
+      in_range[i] = m0 + r0 + 16 * i < M;
+    }
+  }
+  __device__ const bf16* a(int i, int, int k, int, bool& ok) const {
+    ok = in_range[i] && k < LDY;
+    return row[i] + k;
+  }
+  __device__ const bf16* at(int, int, int, int, bool&) const { return nullptr; }
+  __device__ const bf16* b(int, int k, int n, int, int, bool& ok) const {
+    ok = k < NOUT;
+    return w + (int64_t)k * NIN + n;
+  }
+  __device__ void store(int, int m, int n, uint4 v) const {
+    *reinterpret_cast<uint4*>(dx + (int64_t)m * NIN + n) = relu_mask(v, x + (int64_t)m * NIN + n);
+  }
+  __device__ void add(int, int, float) const {}
+};
+// dW[o, i] += sum_b dy[b, o] x[b, i]
+template <int NIN, int NOUT, int LDY>
+struct FcWgrad : SplitK {
+  static constexpr bool A_K = false, SUM = true;
+  static constexpr int BN = 64;
+  const bf16 *dy, *x;
+  float* dw;
+  __device__ const bf16* any() const { return x; }
+  __device__ void rows(int, int, int) {}
+  __device__ const bf16* a(int, int, int, int, bool&) const { return nullptr; }
+  __device__ const bf16* at(int k, int m, int, int ke, bool& ok) const {
+    ok = k < ke && m < LDY;
+    return dy + (int64_t)k * LDY + m;
+  }
+  __device__ const bf16* b(int, int k, int n, int, int ke, bool& ok) const {
+    ok = k < ke;
+    return x + (int64_t)k * NIN + n;
+  }
+  __device__ void add(int m, int n, float v) const { atomicAdd(dw + (int64_t)m * NIN + n, v); }
+  __device__ void store(int, int, int, uint4) const {}
+};
+
+// The last layer's gradient [B][27] in BF16 rows of 32 (zeros after the 27).
+constexpr int LDY6 = 32;
+__global__ void last_grad_kernel(const float* __restrict__ dy, int B, bf16* __restrict__ out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)B * LDY6; i += (int64_t)gridDim.x * blockDim.x) {
+    const int n = (int)(i % LDY6);
+    out[i] = __float2bfloat16(n < NOUT ? dy[i / LDY6 * NOUT + n] : 0.f);
+  }
 }
 
-template <class T>
-cudaError_t bias_grad(const T* g, int64_t rows, int C, float* db, cudaStream_t st) {
-  const int lanes = std::max(1, 256 / C);
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((rows + lanes - 1) / lanes, 1024));
-  bias_grad_kernel<T><<<blocks, lanes * C, 0, st>>>(g, rows, C, db);
-  return cudaGetLastError();
+// First layer's weight gradient, dW[co, kh, kw, ci] += sum_px d[px, co] x[px's window]: the windows are 45 values
+// at a 10-byte stride, so a warp builds them (rows of 48) from the image kept in shared memory, 16 bytes a
+// pixel with a border of zeros, one image row of 32 pixels at a time, and multiplies 32 x 48 blocks; a
+// CTA's warps take every fourth row of its images and add up in shared memory at the end.
+constexpr int W1_IMG_LD = 40, W1_LDB = 56, W1_LDA = 40;
+struct W1Smem {
+  uint4 img[34 * W1_IMG_LD];
+  bf16 Bt[4][32 * W1_LDB], At[4][2][32 * W1_LDA];
+  float sum[C1 * 48];
+};
+__global__ void __launch_bounds__(128) conv1_wgrad_kernel(const bf16* __restrict__ x, const bf16* __restrict__ d, int B,
+                                                          float* __restrict__ dw) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  W1Smem& S = *reinterpret_cast<W1Smem*>(dyn);
+  uint4* const img = S.img;
+  auto& Bt = S.Bt;
+  auto& At = S.At;
+  float* const sum = S.sum;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto at = [](int p) { return p + (p >> 3); };   // a gap after every eighth pixel spreads the writes over the banks
+  for (int i = tid; i < 34 * W1_IMG_LD; i += 128) img[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = tid; i < C1 * 48; i += 128) sum[i] = 0.f;
+  float acc[2][6][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 6; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+  for (int b = blockIdx.x; b < B; b += gridDim.x) {
+    const bf16* dimg = d + (int64_t)b * (IMG * IMG * C1);
+    auto fetch = [&](int q) {   // this warp's q-th row of the image: 32 pixels x 32 channels
+      if (q < 8) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int e = lane + 32 * i, r = e >> 2, c = e & 3;
+          copy16(At[warp][q & 1] + r * W1_LDA + 8 * c, dimg + ((4 * q + warp) * 32 + r) * C1 + 8 * c, true);
+        }
+      }
+      cp_async_commit();
+    };
+    fetch(0);
+    __syncthreads();   // the previous image has been read
+    const uint16_t* src = reinterpret_cast<const uint16_t*>(x) + (int64_t)b * (IMG * IMG * CIN);
+    for (int p = tid; p < IMG * IMG; p += 128) {
+      const uint16_t* s = src + 5 * p;
+      img[((p >> 5) + 1) * W1_IMG_LD + at((p & 31) + 1)] =
+          make_uint4(s[0] | ((uint32_t)s[1] << 16), s[2] | ((uint32_t)s[3] << 16), s[4], 0u);
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int q = 0; q < 8; ++q) {
+      fetch(q + 1);
+      // windows of output row 4 q + warp, lane = column: three runs of 15 values
+      uint32_t r[3][8];
+#pragma unroll
+      for (int kh = 0; kh < 3; ++kh) {
+        const uint4* p = img + (4 * q + warp + kh) * W1_IMG_LD;
+        const uint4 p0 = p[at(lane)], p1 = p[at(lane + 1)], p2 = p[at(lane + 2)];
+        r[kh][0] = p0.x;
+        r[kh][1] = p0.y;
+        r[kh][2] = p0.z | (p1.x << 16);
+        r[kh][3] = __funnelshift_r(p1.x, p1.y, 16);
+        r[kh][4] = __funnelshift_r(p1.y, p1.z, 16);
+        r[kh][5] = p2.x;
+        r[kh][6] = p2.y;
+        r[kh][7] = p2.z;
+      }
+      uint4* o = reinterpret_cast<uint4*>(Bt[warp] + lane * W1_LDB);
+      o[0] = make_uint4(r[0][0], r[0][1], r[0][2], r[0][3]);
+      o[1] = make_uint4(r[0][4], r[0][5], r[0][6], r[0][7] | (r[1][0] << 16));
+      o[2] = make_uint4(__funnelshift_r(r[1][0], r[1][1], 16), __funnelshift_r(r[1][1], r[1][2], 16),
+                        __funnelshift_r(r[1][2], r[1][3], 16), __funnelshift_r(r[1][3], r[1][4], 16));
+      o[3] = make_uint4(__funnelshift_r(r[1][4], r[1][5], 16), __funnelshift_r(r[1][5], r[1][6], 16),
+                        __funnelshift_r(r[1][6], r[1][7], 16), r[2][0]);
+      o[4] = make_uint4(r[2][1], r[2][2], r[2][3], r[2][4]);
+      o[5] = make_uint4(r[2][5], r[2][6], r[2][7], 0u);
+      copy_wait<1>();
+      __syncwarp();
+      const bf16* A = At[warp][q & 1];
+#pragma unroll
+      for (int kk = 0; kk < 32; kk += 16) {
+        uint32_t a[2][4], bb[3][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) frag_at<W1_LDA>(a[i], A, 16 * i, kk, lane);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) frag_b<W1_LDB>(bb[j], Bt[warp], kk, 16 * j, lane);
+#pragma unroll
+        for (int j = 0; j < 6; ++j)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) mma16816(acc[i][j], a[i], bb[j >> 1][2 * (j & 1)], bb[j >> 1][2 * (j & 1) + 1]);
+      }
+      __syncwarp();   // the windows and the row's buffer are rewritten
+    }
+    copy_wait<0>();
+  }
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 6; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) atomicAdd(&sum[(16 * i + g + (e >> 1) * 8) * 48 + 8 * j + 2 * t + (e & 1)], acc[i][j][e]);
+  __syncthreads();
+  for (int i = tid; i < C1 * 9 * CIN; i += 128) atomicAdd(dw + i, sum[i / 45 * 48 + i % 45]);
+}
+
+// Bias gradients of all layers, db[c] += sum over rows of g[r, c]: blockIdx.y is the layer; a thread adds up 8
+// channels of every so many rows, the block its threads.
+struct BiasJob {
+  const bf16* g;       // [rows][C] (null: the FP32 one)
+  const float* gf;
+  int64_t rows;
+  int C;
+  float* db;
+};
+struct BiasJobs {
+  BiasJob j[6];
+};
+__global__ void __launch_bounds__(256) bias_grad_kernel(BiasJobs jobs) {
+  const BiasJob J = jobs.j[blockIdx.y];
+  __shared__ float sum[F5];
+  for (int c = threadIdx.x; c < J.C; c += 256) sum[c] = 0.f;
+  __syncthreads();
+  if (J.g) {
+    const int groups = J.C / 8, c = threadIdx.x % groups, lanes = 256 / groups;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int64_t r = (int64_t)blockIdx.x * lanes + threadIdx.x / groups; r < J.rows; r += (int64_t)gridDim.x * lanes) {
+      const uint4 v = *reinterpret_cast<const uint4*>(J.g + r * J.C + 8 * c);
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        s[2 * i] += __uint_as_float(w[i] << 16);
+        s[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) atomicAdd(&sum[8 * c + i], s[i]);
+  } else {
+    const int lanes = 256 / J.C, c = threadIdx.x % J.C, l = threadIdx.x / J.C;
+    float s = 0.f;
+    if (l < lanes)
+      for (int64_t r = (int64_t)blockIdx.x * lanes + l; r < J.rows; r += (int64_t)gridDim.x * lanes) s += J.gf[r * J.C + c];
+    if (l < lanes) atomicAdd(&sum[c], s);
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < J.C; c += 256) atomicAdd(J.db + c, sum[c]);
 }
 
 // ------------------------------------------------------------------------------ small kernels
@@ -521,42 +903,64 @@ extern "C" int celeste_cnn_backward(const float* params, const uint16_t* params_
   const Ws w = ws_layout(static_cast<char*>(ws), batch);
   const int B = batch;
   const bf16* xin = reinterpret_cast<const bf16*>(x);
-  ConvGeom g1{B, 32, 32, CIN, 32, 32, C1, 1}, g2{B, 32, 32, C1, 16, 16, C2, 2};
-  ConvGeom g3{B, 16, 16, C2, 8, 8, C3, 2}, g4{B, 8, 8, C3, 4, 4, C4, 2};
   cudaError_t e;
-  auto splits_for = [](int64_t K) { return (int)std::max<int64_t>(1, std::min<int64_t>(256, K / 1024)); };
-  // fc2
-  if ((e = gemm(FcWgrad<float>{F5, NOUT, dy, w.a5, grad + o.w6}, NOUT, F5, B, splits_for(B), st)) != cudaSuccess ||
-      (e = bias_grad(dy, B, NOUT, grad + o.b6, st)) != cudaSuccess ||
-      (e = gemm(FcDgrad<float>{F5, NOUT, dy, pb + o.w6, w.a5, w.d5}, B, F5, NOUT, 1, st)) != cudaSuccess)
-    return cuda_fail(e, "cnn backward fc2");
-  // fc1
-  if ((e = gemm(FcWgrad<bf16>{FLAT, F5, w.d5, w.a4, grad + o.w5}, F5, FLAT, B, splits_for(B), st)) != cudaSuccess ||
-      (e = bias_grad(w.d5, B, F5, grad + o.b5, st)) != cudaSuccess ||
-      (e = gemm(FcDgrad<bf16>{FLAT, F5, w.d5, pb + o.w5, w.a4, w.d4}, B, FLAT, F5, 1, st)) != cudaSuccess)
-    return cuda_fail(e, "cnn backward fc1");
-  // conv4 .. conv1
-  struct L {
-    ConvGeom g;
-    const bf16* in;
-    const bf16* d;
-    bf16* din;
-    int64_t w, b;
-  } layers[4] = {{g4, w.a3, w.d4, w.d3, o.w4, o.b4},
-                 {g3, w.a2, w.d3, w.d2, o.w3, o.b3},
-                 {g2, w.a1, w.d2, w.d1, o.w2, o.b2},
-                 {g1, xin, w.d1, nullptr, o.w1, o.b1}};
-  for (const L& l : layers) {
-    const int64_t Kw = (int64_t)l.g.B * l.g.OH * l.g.OW;
-    if ((e = gemm(ConvWgrad{l.g, l.d, l.in, grad + l.w}, l.g.Cout, 9 * l.g.Cin, (int)Kw, splits_for(Kw), st)) !=
-            cudaSuccess ||
-        (e = bias_grad(l.d, Kw, l.g.Cout, grad + l.b, st)) != cudaSuccess)
-      return cuda_fail(e, "cnn backward weights");
-    if (l.din &&
-        (e = gemm(ConvDgrad{l.g, l.d, pb + l.w, l.in, l.din}, l.g.B * l.g.H * l.g.W, l.g.Cin, 9 * l.g.Cout, 1, st)) !=
-            cudaSuccess)
-      return cuda_fail(e, "cnn backward data");
-  }
+  int dev = 0, n_sm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return cuda_fail(e, "SM count");
+  // K split of a weight gradient: about four CTAs per SM, each with at least four K-steps
+  auto chunk_for = [n_sm](int tiles, int K) {
+    const int want = std::max(1, (4 * n_sm + tiles - 1) / tiles);
+    return std::max(4 * BK2, (K / want + BK2 - 1) / BK2 * BK2);
+  };
+  auto wgrad = [&](const auto& op, int M, int N, int K) {
+    const int chunk = chunk_for((M + 63) / 64 * ((N + 63) / 64), K);
+    return bwd_gemm(op, M, N, K, (K + chunk - 1) / chunk, chunk, st);
+  };
+  // The last layer's gradient in BF16 goes to the first layer's gradient buffer, which is written last.
+  bf16* dy6 = w.d1;
+  last_grad_kernel<<<(int)std::min<int64_t>(((int64_t)B * LDY6 + 255) / 256, 4 * n_sm), 256, 0, st>>>(dy, B, dy6);
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "cnn backward output gradient");
+  FcWgrad<F5, NOUT, LDY6> w6{};
+  w6.dy = dy6, w6.x = w.a5, w6.dw = grad + o.w6;
+  FcDgrad<F5, NOUT, LDY6> d6{};
+  d6.dy = dy6, d6.w = pb + o.w6, d6.x = w.a5, d6.dx = w.d5;
+  FcWgrad<FLAT, F5, F5> w5{};
+  w5.dy = w.d5, w5.x = w.a4, w5.dw = grad + o.w5;
+  FcDgrad<FLAT, F5, F5> d5{};
+  d5.dy = w.d5, d5.w = pb + o.w5, d5.x = w.a4, d5.dx = w.d4;
+  if ((e = wgrad(w6, NOUT, F5, B)) != cudaSuccess || (e = bwd_gemm(d6, B, F5, LDY6, 1, LDY6, st)) != cudaSuccess ||
+      (e = wgrad(w5, F5, FLAT, B)) != cudaSuccess || (e = bwd_gemm(d5, B, FLAT, F5, 1, F5, st)) != cudaSuccess)
+    return cuda_fail(e, "cnn backward dense layers");
+  ConvWgrad<4, C3> w4{};
+  w4.dout = w.d4, w4.in = w.a3, w4.dw = grad + o.w4;
+  ConvDgrad<4, C3> d4{};
+  d4.dout = w.d4, d4.w = pb + o.w4, d4.in = w.a3, d4.din = w.d3;
+  ConvWgrad<8, C2> w3{};
+  w3.dout = w.d3, w3.in = w.a2, w3.dw = grad + o.w3;
+  ConvDgrad<8, C2> d3{};
+  d3.dout = w.d3, d3.w = pb + o.w3, d3.in = w.a2, d3.din = w.d2;
+  ConvWgrad<16, C1> w2{};
+  w2.dout = w.d2, w2.in = w.a1, w2.dw = grad + o.w2;
+  ConvDgrad<16, C1> d2{};
+  d2.dout = w.d2, d2.w = pb + o.w2, d2.in = w.a1, d2.din = w.d1;
+  if ((e = wgrad(w4, C4, 9 * C3, B * 16)) != cudaSuccess || (e = bwd_gemm(d4, B * 16, C3, 256, 4, 0, st)) != cudaSuccess ||
+      (e = wgrad(w3, C3, 9 * C2, B * 64)) != cudaSuccess || (e = bwd_gemm(d3, B * 64, C2, 256, 4, 0, st)) != cudaSuccess ||
+      (e = wgrad(w2, C2, 9 * C1, B * 256)) != cudaSuccess || (e = bwd_gemm(d2, B * 256, C1, 256, 4, 0, st)) != cudaSuccess)
+    return cuda_fail(e, "cnn backward convolutions");
+  if ((e = cudaFuncSetAttribute(conv1_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(W1Smem))) !=
+      cudaSuccess)
+    return cuda_fail(e, "cnn backward first layer");
+  conv1_wgrad_kernel<<<std::min(B, 2 * n_sm), 128, sizeof(W1Smem), st>>>(xin, w.d1, B, grad + o.w1);
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "cnn backward first layer");
+  const BiasJobs jobs = {{{w.d1, nullptr, (int64_t)B * 1024, C1, grad + o.b1},
+                          {w.d2, nullptr, (int64_t)B * 256, C2, grad + o.b2},
+                          {w.d3, nullptr, (int64_t)B * 64, C3, grad + o.b3},
+                          {w.d4, nullptr, (int64_t)B * 16, C4, grad + o.b4},
+                          {w.d5, nullptr, (int64_t)B, F5, grad + o.b5},
+                          {nullptr, dy, (int64_t)B, NOUT, grad + o.b6}}};
+  bias_grad_kernel<<<dim3(std::min(n_sm, B), 6), 256, 0, st>>>(jobs);
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "cnn backward biases");
   return CELESTE_OK;
 }
 
