@@ -505,30 +505,60 @@ __global__ void __launch_bounds__(32 * NW) assemble_kernel(ProblemDev P, const d
 }
 
 // Value-only assembly, one warp per source: sum of the value tile sums minus the KL at theta
-// (plus the KL at theta_ref when the pixel sums are differences from theta_ref).
+// (plus the KL at theta_ref when the pixel sums are differences from theta_ref).  A chain of latencies: the
+// patches' tile ranges and then their tiles are loaded for up to 32 patches at once, and one
+// exponential serves the log-variances and both type probabilities (one source 10.9 us per launch, cold, with a
+// patch after the other; 8.4 now).
 __global__ void assemble_value_kernel(ProblemDev P, const double* __restrict__ theta, const double* __restrict__ theta_ref,
                                       double* out) {
   const int lane = threadIdx.x & 31;
   for (int s = wl_next_warp(P, WL_SOURCES); s >= 0; s = wl_next_warp(P, WL_SOURCES)) {   // warp-uniform
-  double v = 0.0;
-  for (int p = P.src_patch[s]; p < P.src_patch[s + 1]; ++p) {
-    const PatchDev& pt = P.patches[p];
-    for (int t = pt.tile_begin + lane; t < pt.tile_end; t += 32) v += (double)P.vpartials[t];
-  }
   // KL terms: lanes 0..10 at theta, lanes 16..26 at theta_ref (subtracted / added)
   const int which = lane >> 4, k = lane & 15;
   const double* th = which ? theta_ref : theta;
+  double al = 0.0, x = 0.0;
+  const int t = k / 5, kk = k % 5;   // (k < 10)
+  if (th) {
+    th += (size_t)s * NP;
+    al = th[6];
+    x = k < 10 ? th[bvar(t, kk == 0 ? 1 : 5 + kk)] : -fabs(al);
+  }
+  double v = 0.0;
+  const int p0 = P.src_patch[s], p1 = P.src_patch[s + 1];
+  for (int pb = p0; pb < p1; pb += 32) {
+    const int n = min(32, p1 - pb);
+    int tb = 0, te = 0;
+    if (lane < n) {
+      tb = P.patches[pb + lane].tile_begin;
+      te = P.patches[pb + lane].tile_end;
+    }
+    for (int q0 = 0; q0 < n; q0 += 4) {
+      // the first 32 tiles of four patches at once, the rest of a patch after them
+      float x0[4];
+      int b[4], e[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        b[i] = __shfl_sync(0xffffffffu, tb, (q0 + i) & 31);
+        e[i] = q0 + i < n ? __shfl_sync(0xffffffffu, te, (q0 + i) & 31) : 0;
+        x0[i] = b[i] + lane < e[i] ? P.vpartials[b[i] + lane] : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (b[i] + lane < e[i]) v += (double)x0[i];
+        for (int u = b[i] + 32 + lane; u < e[i]; u += 32) v += (double)P.vpartials[u];
+      }
+    }
+  }
+  const double ex = th && k <= 10 ? exp(x) : 0.0;
+  const double em = __shfl_sync(0xffffffffu, ex, (lane & 16) + 10);   // exp(-|alpha|)
   if (th && k <= 10) {
-    th += (size_t)s * NP;   // (per-lane pointer; th is reset each source)
-    const double al = th[6], e = exp(-fabs(al)), sg = 1.0 / (1.0 + e);
-    const double a1 = al >= 0 ? sg : e * sg, a0 = al >= 0 ? e * sg : sg;
+    const double sg = 1.0 / (1.0 + em);
+    const double a1 = al >= 0 ? sg : em * sg, a0 = al >= 0 ? em * sg : sg;
     double klp;
     if (k < 10) {
-      const int t = k / 5, kk = k % 5;
-      const double ev = exp(th[bvar(t, kk == 0 ? 1 : 5 + kk)]);
-      klp = (t ? a1 : a0) * kl_normal_term(th, ev, P, t, kk);
+      klp = (t ? a1 : a0) * kl_normal_term(th, ex, P, t, kk);
     } else {
-      const double l1p = log1p(e);
+      const double l1p = log1p(em);
       const double la1 = al >= 0 ? -l1p : al - l1p, la0 = la1 - al;
       klp = a1 * (la1 - P.log_phi) + a0 * (la0 - P.log1m_phi);
     }

@@ -279,10 +279,14 @@ __global__ void tr_reciprocal_kernel(const double* __restrict__ x, double* __res
   if (i < n) r[i] = tr_rcp(x[i]);
 }
 
-// Accept or reject the trial point and update the radius (Nocedal & Wright Alg. 4.1).
-__global__ void tr_update_kernel(NewtonDev N, int* flags) {
+// Accept or reject the trial point and update the radius (Nocedal & Wright Alg. 4.1).  One thread per
+// source decides; the accepted points are copied by the whole warp, one source's 27 numbers at a time (32
+// threads each walking their own row took twice as long).
+constexpr int UPDATE_THREADS = 32;
+__global__ void __launch_bounds__(UPDATE_THREADS) tr_update_kernel(NewtonDev N, int* flags) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   int active = 0;
+  bool accepted = false;
   if (s < N.S) {
     int* st = N.state + ST_STRIDE * s;
     if (flags[s] & FLAG_VALUE) {
@@ -308,7 +312,7 @@ __global__ void tr_update_kernel(NewtonDev N, int* flags) {
           st[ST_CACHED] = 0;
           const double Lnew = N.L[s] + dL;
           const bool done = fabs(dL) <= N.ftol * fabs(Lnew);
-          for (int k = 0; k < NP; ++k) N.theta[(size_t)s * NP + k] = N.trial[(size_t)s * NP + k];
+          accepted = true;
           N.L[s] = Lnew;
           if (done) {
             st[ST_ACTIVE] = 0;
@@ -329,9 +333,13 @@ __global__ void tr_update_kernel(NewtonDev N, int* flags) {
     }
     active = st[ST_ACTIVE];
   }
+  const int lane = threadIdx.x & 31;
+  for (unsigned todo = __ballot_sync(0xffffffffu, accepted); todo; todo &= todo - 1) {
+    const size_t o = (size_t)(s - lane + __ffs(todo) - 1) * NP + lane;
+    if (lane < NP) N.theta[o] = N.trial[o];
+  }
   // count and list the active sources (one atomic per warp)
   const unsigned m = __ballot_sync(0xffffffffu, active);
-  const int lane = threadIdx.x & 31;
   int base = 0;
   if (lane == 0 && m) base = atomicAdd(N.count, __popc(m));
   base = __shfl_sync(0xffffffffu, base, 0);
@@ -376,7 +384,7 @@ static cudaError_t newton_iteration(const ProblemDev& D, const NewtonDev& N, cud
   if ((e = mark(1)) != cudaSuccess) return e;
   if ((e = launch_assemble_value(D, N.trial, N.theta, N.Ltrial, st)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(N.count, 0, sizeof(int), st)) != cudaSuccess) return e;
-  tr_update_kernel<<<(S + 127) / 128, 128, 0, st>>>(N, D.flags);
+  tr_update_kernel<<<(S + UPDATE_THREADS - 1) / UPDATE_THREADS, UPDATE_THREADS, 0, st>>>(N, D.flags);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_worklists(D, FLAG_FULL, st)) != cudaSuccess) return e;
   if ((e = launch_tables(D, N.theta, true, st)) != cudaSuccess) return e;
