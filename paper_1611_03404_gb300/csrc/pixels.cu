@@ -437,15 +437,6 @@ struct PixGeo {
   }
 };
 
-// 2^x by the special-function unit alone, subnormal results as 0: what that leaves out is under
-// 1.2e-38, where the rate it is added to is at least the sky's.  (exp2f spends three more
-// instructions per component on those subnormals: 4 % of the kernel.)
-__device__ __forceinline__ float ex2_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // One galaxy mixture component's value at a pixel (e: its table entry).
 __device__ __forceinline__ float gal_value(const float (&e)[GT_STRIDE], const PixGeo& g) {
   const float q = fmaf(e[GT_P + 2], g.S2.x, fmaf(e[GT_P + 1], g.S1.x, e[GT_P] * g.S0.x));
@@ -887,7 +878,7 @@ __global__ void __launch_bounds__(BLOCK) elbo_value_kernel(ProblemDev P, int dif
         const float4 a = vp[2 * pr], w = vp[2 * pr + 1];   // (P00, P00', P01, P01'), (P11, P11', W, W')
         const float2 q = fma2(f2(w.x, w.y), S2, fma2(f2(a.z, a.w), S1, mul2(f2(a.x, a.y), S0)));
         const float2 qs = mul2(q, f2(-0.5f * LOG2E, -0.5f * LOG2E));
-        const float2 g = mul2(f2(w.z, w.w), f2(exp2f(qs.x), exp2f(qs.y)));
+        const float2 g = mul2(f2(w.z, w.w), f2(ex2_ftz(qs.x), ex2_ftz(qs.y)));
         if (pr < CELESTE_NEXP / 2)
           fE = add2(fE, g);
         else
