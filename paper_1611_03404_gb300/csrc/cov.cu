@@ -3,20 +3,24 @@
 // solver's exact Hessian): Sigma = (-H)^-1, where H is the ELBO Hessian w.r.t. the 27 free
 // parameters.  Defined only where -H is positive definite (a strict local maximum).
 //
-// One warp per source, float64: -H = L D L^T in place (lane i owns row i), then the 27 columns of
-// the inverse solved at once, lane j carrying the right-hand side e_j (a float64 warp instruction
-// costs the same for 1 or 32 lanes on this part, so the 27 solves cost one).
+// One warp per source, float64: -H = L D L^T in place, then the 27 columns of the inverse solved at once.
+// A float64 warp instruction costs the same for 1 or 32 lanes on this part and bounds the kernel, so the
+// factorisation's updates and the forward solve, whose right-hand sides are unit vectors (column j starts at
+// row j), deal their entries to the lanes one by one; the backward solve has a column per lane.  1000 sources
+// 82 us with a row or column per lane throughout, 71 now.
 #include <algorithm>
 
 #include "celeste_internal.cuh"
 #include "kernels.h"
 #include "problem.h"
+#include "trsolve.cuh"
 
 namespace celeste {
 
 struct CovSmem {
   double A[NP * NP];     // -H, then L below the diagonal
   double r[NP];          // reciprocal pivots
+  double l[32];          // a step's column of L
   double Y[NP][32];      // lane j: the solve for e_j
 };
 
@@ -34,14 +38,19 @@ __global__ void __launch_bounds__(32) cov_kernel(const double* __restrict__ H, i
     pd = dk > 0.0 && isfinite(dk);   // same value in every lane
     if (!pd) break;
     const double rk = 1.0 / dk;
-    const bool act = lane > k && lane < NP;
-    const double li = act ? sm.A[lane * NP + k] * rk : 0.0;
-    __syncwarp();
-    if (act) {
-      for (int j = k + 1; j < NP; ++j) sm.A[lane * NP + j] = fma(-li, sm.A[k * NP + j], sm.A[lane * NP + j]);
+    if (lane > k && lane < NP) {
+      const double li = sm.A[lane * NP + k] * rk;
+      sm.l[lane] = li;
       sm.A[lane * NP + k] = li;
     }
     if (lane == 0) sm.r[k] = rk;
+    __syncwarp();
+    const int m = NP - 1 - k;
+    if (m > 0) {
+      const double *l = sm.l + k + 1, *rw = sm.A + k * NP + k + 1;
+      double* T = sm.A + (k + 1) * NP + k + 1;
+      for (TrWalk q(lane, 32, m); q.i < m; q.next()) T[q.i * NP + q.j] = fma(-l[q.i], rw[q.j], T[q.i * NP + q.j]);
+    }
     __syncwarp();
   }
   if (lane == 0) ok[s] = pd ? 1 : 0;
@@ -50,13 +59,18 @@ __global__ void __launch_bounds__(32) cov_kernel(const double* __restrict__ H, i
     for (int i = lane; i < NP * NP; i += 32) out[i] = __longlong_as_double(0x7ff8000000000000LL);
     return;
   }
-  // lane j < 27: L y = e_j, y *= D^-1, L^T x = y
-  if (lane < NP) {
-    for (int i = 0; i < NP; ++i) {
-      double acc = i == lane ? 1.0 : 0.0;
-      for (int k = 0; k < i; ++k) acc = fma(-sm.A[i * NP + k], sm.Y[k][lane], acc);
-      sm.Y[i][lane] = acc;
+  // L Y = I: step k takes L_ik Y_kj off Y_ij for i > k, j <= k
+  for (int i = 0; i < NP; ++i) sm.Y[i][lane] = i == lane ? 1.0 : 0.0;
+  __syncwarp();
+  for (int k = 0; k < NP - 1; ++k) {
+    for (TrWalk q(lane, 32, k + 1); q.i < NP - 1 - k; q.next()) {
+      const int i = k + 1 + q.i;
+      sm.Y[i][q.j] = fma(-sm.A[i * NP + k], sm.Y[k][q.j], sm.Y[i][q.j]);
     }
+    __syncwarp();
+  }
+  // lane j < 27: y *= D^-1, L^T x = y
+  if (lane < NP) {
     for (int i = 0; i < NP; ++i) sm.Y[i][lane] *= sm.r[i];
     for (int i = NP - 2; i >= 0; --i) {
       double acc = sm.Y[i][lane];
