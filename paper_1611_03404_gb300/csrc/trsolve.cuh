@@ -8,7 +8,7 @@
 // FP64 pipe of an SM sub-partition retires a warp-wide FMA only every several tens of cycles), so
 // the solver keeps that count low:
 //   * Newton step first: where the caller expects it (the previous step was interior), B is
-//     factored B = L D L^T in place (lane i owns row i); if every pivot is positive and
+//     factored B = L D L^T in place (updates dealt entry by entry); if every pivot is positive and
 //     |B^-1 g| <= delta the Newton step is the solution and nothing else runs;
 //   * otherwise B is reduced once to tridiagonal form T = Q^T B Q by Householder reflections
 //     (lane-parallel; g is reflected in the same reductions), after which every solve with
