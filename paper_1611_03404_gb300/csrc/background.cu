@@ -168,6 +168,11 @@ cudaError_t launch_background(const ProblemDev& P, const double* nbr_theta, int 
   if (e == cudaSuccess) e = launch_worklists(P, FLAG_VALUE, st);
   if (e == cudaSuccess) e = launch_tables(P, nbr_theta, false, st);
   if (e != cudaSuccess) return e;
+  return launch_background_kernel(P, clip, st);
+}
+
+cudaError_t launch_background_kernel(const ProblemDev& P, int clip, cudaStream_t st) {
+  if (P.n_tiles == 0) return cudaSuccess;
   // Tiles per CTA: more than one only where 32 CTAs per SM are left, at most eight (2000 sources of wide
   // patches: one tile 2121 us, eight 1863, sixteen the same).
   const int group = std::max(1, std::min(8, P.n_tiles / (P.n_sm * 32))), g = (P.n_tiles + group - 1) / group;

@@ -7,6 +7,8 @@ namespace celeste {
 
 // clip: neighbours counted on their own windows only (the joint objective's per-source blocks).
 cudaError_t launch_background(const ProblemDev& P, const double* nbr_theta, int clip, cudaStream_t st);
+// The background of every tile alone, on tables already built for all patches.
+cudaError_t launch_background_kernel(const ProblemDev& P, int clip, cudaStream_t st);
 // Rebuilds the tile/patch/source worklists from the sources whose flags match `mask`. Every
 // launcher below works on the current worklists, whose counts live on the device, so a sequence
 // of launches needs no host round trip and can be captured in a CUDA graph.
@@ -15,10 +17,8 @@ cudaError_t launch_worklists(const ProblemDev& P, int mask, cudaStream_t st);
 cudaError_t launch_tables(const ProblemDev& P, const double* theta, bool full, cudaStream_t st);
 // Tables (full) + ELBO/gradient/Hessian tile sums for the listed tiles.
 cudaError_t launch_full(const ProblemDev& P, const double* theta, cudaStream_t st);
-// Tables (value) + value-only tile sums for the listed tiles (diff: differences from the stored
+// The pixel kernels alone, on tables already built for the listed patches (diff: differences from the stored
 // per-pixel source moments).
-cudaError_t launch_value(const ProblemDev& P, const double* theta, bool diff, cudaStream_t st);
-// The pixel kernels alone, on tables already built for the listed patches.
 cudaError_t launch_full_kernel(const ProblemDev& P, cudaStream_t st);
 cudaError_t launch_value_kernel(const ProblemDev& P, bool diff, cudaStream_t st);
 // Per-source float64 sum of the value-only tile sums minus the KL at theta; with theta_ref the

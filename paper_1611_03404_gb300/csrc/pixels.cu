@@ -960,13 +960,6 @@ cudaError_t launch_full_kernel(const ProblemDev& P, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_value(const ProblemDev& P, const double* theta, bool diff, cudaStream_t st) {
-  if (P.n_tiles == 0) return cudaSuccess;
-  cudaError_t e = launch_tables(P, theta, false, st);
-  if (e != cudaSuccess) return e;
-  return launch_value_kernel(P, diff, st);
-}
-
 cudaError_t launch_value_kernel(const ProblemDev& P, bool diff, cudaStream_t st) {
   if (P.n_tiles == 0) return cudaSuccess;
   const int d = diff ? (P.refEV ? 2 : 1) : 0;   // difference from the joint reference rates when set
