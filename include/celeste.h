@@ -439,6 +439,14 @@ int celeste_cnn_forward_ex(const float* params, const uint16_t* params_bf16, con
                            const float* out_scale, const float* out_shift, float* y, void* ws, size_t ws_bytes,
                            int engine, celeste_stream_t stream);
 
+/* celeste_cnn_forward_ex with the budget, in SM clock cycles, of each of the tcgen05 kernels' waits (0: the
+ * default, ~2 s; a negative budget makes every wait give up at once, without waiting).  Where a wait runs
+ * out the outputs are undefined, celeste_cnn_status reports it, and the device stays usable: the tests
+ * reach the timeout path this way. */
+int celeste_cnn_forward_budget(const float* params, const uint16_t* params_bf16, const uint16_t* x, int batch,
+                               const float* out_scale, const float* out_shift, float* y, void* ws, size_t ws_bytes,
+                               int engine, long long wait_budget, celeste_stream_t stream);
+
 /* CELESTE_ERR_TIMEOUT (and clears it) if a tensor-core product of the network's forward pass did not
  * complete within its wait budget since the last call; CELESTE_OK otherwise.  Synchronous (reads a
  * device word of the current device). */

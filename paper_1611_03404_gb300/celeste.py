@@ -60,7 +60,7 @@ EXPORTED = ["celeste_problem_create", "celeste_problem_workspace_bytes", "celest
             "celeste_render_background_mode", "celeste_joint_pairs", "celeste_joint_cross_hessian",
             "celeste_joint_newton", "celeste_joint_value", "celeste_problem_check", "celeste_problem_set_wait_budget",
             "celeste_measure_peak", "celeste_joint_workspace_bytes", "celeste_joint_bind", "celeste_cnn_forward_ex",
-            "celeste_cnn_status", "celeste_problem_refresh_pixels"]
+            "celeste_cnn_status", "celeste_problem_refresh_pixels", "celeste_cnn_forward_budget"]
 
 
 def load_library(path=None):
@@ -107,6 +107,8 @@ def load_library(path=None):
         "celeste_joint_workspace_bytes": (ctypes.c_size_t, [vp]),
         "celeste_cnn_forward_ex": (ctypes.c_int, [dp, dp, dp, ctypes.c_int, dp, dp, dp, dp, ctypes.c_size_t,
                                                   ctypes.c_int, vp]),
+        "celeste_cnn_forward_budget": (ctypes.c_int, [dp, dp, dp, ctypes.c_int, dp, dp, dp, dp, ctypes.c_size_t,
+                                                      ctypes.c_int, ctypes.c_longlong, vp]),
         "celeste_cnn_status": (ctypes.c_int, []),
         "celeste_problem_refresh_pixels": (ctypes.c_int, [vp, vp]),
         "celeste_joint_bind": (ctypes.c_int, [vp, vp, ctypes.c_size_t, vp]),

@@ -841,6 +841,14 @@ extern "C" int celeste_cnn_forward(const float* params, const uint16_t* params_b
 extern "C" int celeste_cnn_forward_ex(const float* params, const uint16_t* params_bf16, const uint16_t* x, int batch,
                                       const float* out_scale, const float* out_shift, float* y, void* ws,
                                       size_t ws_bytes, int engine, celeste_stream_t stream) {
+  return celeste_cnn_forward_budget(params, params_bf16, x, batch, out_scale, out_shift, y, ws, ws_bytes, engine, 0,
+                                    stream);
+}
+
+extern "C" int celeste_cnn_forward_budget(const float* params, const uint16_t* params_bf16, const uint16_t* x,
+                                          int batch, const float* out_scale, const float* out_shift, float* y,
+                                          void* ws, size_t ws_bytes, int engine, long long wait_budget,
+                                          celeste_stream_t stream) {
   if (!params || !params_bf16 || !x || !y) return fail(CELESTE_ERR_INVALID_ARG, "null argument");
   if ((out_scale == nullptr) != (out_shift == nullptr)) return fail(CELESTE_ERR_INVALID_ARG, "scale and shift go together");
   if (engine != CELESTE_CNN_MMA_SYNC && engine != CELESTE_CNN_TCGEN05)
@@ -868,6 +876,7 @@ extern "C" int celeste_cnn_forward_ex(const float* params, const uint16_t* param
       cnn_tc::Args a{};
       a.M = m, a.N = n, a.B = B;
       a.in = in, a.w = pb + wo, a.bias = params + bo, a.out = out, a.out_f = outf, a.err = err;
+      a.wait_budget = wait_budget ? wait_budget : WAIT_BUDGET_DEFAULT;
       if (outf) a.scale = out_scale, a.shift = out_shift;
       return tc_forward(id, a, n_sm, st);
     };

@@ -27,9 +27,10 @@
 // layer); copies through L1 instead of L2 alone were 4 % slower.  20,000 patches, whole forward: 8.58 ms with
 // element gathers between every two products, 1.38 ms now; one patch 59 us, 75 before.
 //
-// Every wait on an mbarrier is bounded; a role whose wait runs out records it in the error word and leaves
-// its loop, the others' waits then run out as well, and the CTA waits (bounded) for its products in
-// flight before it frees its tensor memory.
+// Every wait on an mbarrier is bounded (Args::wait_budget); a warp whose wait runs out records it in the
+// error word and leaves its loop, all lanes together, the others' waits then run out as well, and the
+// CTA waits (bounded) for its products in flight before it frees its tensor memory.  The first layer's
+// producers, which also meet at barriers without a bound, go on meeting there until the last image.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -92,6 +93,16 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 
 __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// A wait of one thread, bounded by the call's budget (negative: gives up without waiting).
+__device__ __forceinline__ bool wait_thread(const Args& a, uint64_t* bar, uint32_t parity) {
+  return a.wait_budget >= 0 && mbar_wait(bar, parity, a.wait_budget);
+}
+// The same of a whole warp: every lane gives up if one does (the lanes read the clock on their own, and what
+// follows a wait needs the warp together).
+__device__ __forceinline__ bool wait_warp(const Args& a, uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, wait_thread(a, bar, parity));
+}
 
 // One arrival for the whole warp (32 would be served one after the other).
 __device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar) {
@@ -193,7 +204,7 @@ __device__ __forceinline__ bool produce(const Args& a, unsigned char* stages, Ba
     const int m0 = (t / n_cols) * TM, n0 = (t % n_cols) * L::NT;
     const int left = a.M - m0;   // rows of the tile that exist
     const int s = issue.stage();
-    if (!mbar_wait(&bar.empty[s], issue.parity() ^ 1u, WAIT_BUDGET_DEFAULT)) return false;
+    if (!wait_warp(a, &bar.empty[s], issue.parity() ^ 1u)) return false;
     const uint32_t As = smem_u32(stages + s * L::STAGE);
     if constexpr (L::CONV) {
       constexpr int OW = L::OUT_W, RPI = OW * OW, ROW = L::IN_W * L::CIN;   // output pixels per image, input row
@@ -242,7 +253,8 @@ __device__ __forceinline__ bool produce(const Args& a, unsigned char* stages, Ba
 // First layer: image by image.  The image lies in shared memory with its five channels in 16 bytes per
 // pixel and a border of zeros.  Each warp builds whole tiles (four output rows, a lane one column of
 // them, its window's input rows moving through registers), every fourth one; the next image's pixels are
-// loaded into registers (8 per thread) while the current one's tiles are built.
+// loaded into registers (8 per thread) while the current one's tiles are built.  The four warps meet at two
+// barriers per image: one whose wait has run out builds nothing more, but keeps meeting the others.
 template <class L>
 __device__ __forceinline__ bool produce_first(const Args& a, unsigned char* stages, unsigned char* img, Bars& bar, int images) {
   static_assert(L::STAGES == 4, "a warp's tiles go through one stage");
@@ -287,6 +299,7 @@ __device__ __forceinline__ bool produce_first(const Args& a, unsigned char* stag
   Ring<L::STAGES> ring;
   ring.step = warp;
   unsigned char* As = stages + warp * L::STAGE;
+  bool ok = true;   // the same in every lane of a warp
   fetch(blockIdx.x);
   for (int b = blockIdx.x; b < images; b += gridDim.x) {
     producers_sync();   // the previous image has been read (the border zeroed)
@@ -304,11 +317,12 @@ __device__ __forceinline__ bool produce_first(const Args& a, unsigned char* stag
     producers_sync();
     fetch(b + gridDim.x);
 #pragma unroll 1
-    for (int q = warp; q < 8; q += 4) {
+    for (int q = warp; q < 8 && ok; q += 4) {
       uint32_t r0[8], r1[8], r2[8];
       load_row(4 * q - 1, r0);
       load_row(4 * q, r1);
-      if (!mbar_wait(&bar.empty[warp], ring.parity() ^ 1u, WAIT_BUDGET_DEFAULT)) return false;
+      ok = wait_warp(a, &bar.empty[warp], ring.parity() ^ 1u);
+      if (!ok) break;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         load_row(4 * q + j + 1, r2);
@@ -334,22 +348,23 @@ __device__ __forceinline__ bool produce_first(const Args& a, unsigned char* stag
       ring.step += 4;
     }
   }
-  return true;
+  return ok;
 }
 
 // ---------------------------------------------------------------------------------- products
 template <class L>
-__device__ __forceinline__ bool multiply(unsigned char* weights, unsigned char* stages, Bars& bar, uint32_t tmem, int n_mine) {
+__device__ __forceinline__ bool multiply(const Args& a, unsigned char* weights, unsigned char* stages, Bars& bar, uint32_t tmem,
+                                         int n_mine) {
   const uint32_t idesc = instr_desc_bf16(L::NT);
   Ring<L::STAGES> ring;
   for (int q = 0; q < n_mine; ++q) {
     const int acc = q & 1;
-    if (!mbar_wait(&bar.tempty[acc], ((q >> 1) & 1u) ^ 1u, WAIT_BUDGET_DEFAULT)) return false;
+    if (!wait_thread(a, &bar.tempty[acc], ((q >> 1) & 1u) ^ 1u)) return false;
     fence_after_sync();
     const uint32_t d = tmem + (uint32_t)(acc * L::NT);
     for (int ks = 0; ks < L::KSTEPS; ++ks) {
       const int s = ring.stage();
-      if (!mbar_wait(&bar.full[s], ring.parity(), WAIT_BUDGET_DEFAULT)) return false;
+      if (!wait_thread(a, &bar.full[s], ring.parity())) return false;
       fence_after_sync();
       const uint32_t ab = smem_u32(stages + s * L::STAGE);
       const uint32_t bb = L::RESIDENT ? smem_u32(weights + ks * L::B_BYTES) : ab + A_BYTES;
@@ -379,7 +394,7 @@ __device__ __forceinline__ bool finish(const Args& a, unsigned char* staging, co
     if (t >= n_tiles) break;
     const int acc = q & 1;
     const int row0 = (t / n_cols) * TM + 32 * quad, n0 = (t % n_cols) * L::NT;
-    if (!mbar_wait(&bar.tfull[acc], (q >> 1) & 1u, WAIT_BUDGET_DEFAULT)) return false;
+    if (!wait_warp(a, &bar.tfull[acc], (q >> 1) & 1u)) return false;
     fence_after_sync();
     float v[L::NT];
     const uint32_t src = tmem + (uint32_t)(acc * L::NT) + ((uint32_t)(32 * quad) << 16);
@@ -497,7 +512,7 @@ __global__ void __launch_bounds__(THREADS, L::CTAS) tc_layer_kernel(Args a, int 
     cp_async_wait_all();
   } else if (warp == 4) {
     if ((tid & 31) == 0) {
-      ok = multiply<L>(weights, stages, bar, tmem, n_mine);
+      ok = multiply<L>(a, weights, stages, bar, tmem, n_mine);
       mma_commit(&bar.done);   // every product issued so far
       ok = mbar_wait(&bar.done, 0u, WAIT_BUDGET_DEFAULT) && ok;
     }

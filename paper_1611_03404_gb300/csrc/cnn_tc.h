@@ -23,6 +23,7 @@ struct Args {
   const float* scale;
   const float* shift;
   int* err;                      // error word, set when a bounded wait runs out
+  long long wait_budget;         // SM cycles a wait may take (negative: every wait gives up at once)
 };
 
 }  // namespace cnn_tc
