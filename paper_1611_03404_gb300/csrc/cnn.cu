@@ -232,7 +232,8 @@ struct FcFwd {
 constexpr int BK2 = 64, LD2 = 72, STAGES2 = 3;     // rows of 64 values, 16 bytes apart from a multiple of 128
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// 16 bytes global -> shared, asynchronously; zeros where !ok (the source is then not read).
+// 16 bytes global -> shared, asynchronously; zeros where !ok (the source is then not read, but has to lie on a
+// 16-byte boundary all the same: the operations' any() is an address in the workspace).
 __device__ __forceinline__ void copy16(void* dst, const void* src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
@@ -406,7 +407,7 @@ struct ConvDgrad {
   int pi, pj;
   const bf16* row[4];
   int edge[4];   // 1: no output below, 2: none to the right, 4: no row at all
-  __device__ const bf16* any() const { return w; }
+  __device__ const bf16* any() const { return dout; }
   __device__ void range(int z, int, int, int& kb, int& ke) {
     pi = z >> 1;
     pj = z & 1;
@@ -491,7 +492,7 @@ struct FcDgrad : SplitK {
   bf16* dx;
   const bf16* row[4];
   bool in_range[4];
-  __device__ const bf16* any() const { return w; }
+  __device__ const bf16* any() const { return dy; }
   __device__ void rows(int m0, int r0, int M) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
