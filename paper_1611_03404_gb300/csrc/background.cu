@@ -5,6 +5,7 @@
 // clip = 1 (the joint objective's per-source blocks): a neighbour counts only on the pixels of its
 // own window, as every source does in the objective over all sources jointly.
 #include <algorithm>
+#include <type_traits>
 
 #include "celeste_internal.cuh"
 #include "kernels.h"
@@ -43,6 +44,7 @@ __global__ void __launch_bounds__(BLOCK, 12) background_kernel(ProblemDev P, int
   const int t_end = min(P.n_tiles, (int)(blockIdx.x + 1) * group);
   int patch = -1;       // the patch whose records are loaded
   bool staged = false;  // all of its neighbours are in nbs
+  bool wide = false;    // some staged neighbour is (wide_range); the others' sums are the same either way
   PatchDev pt;
   float sky = 0.f, iota = 0.f;
   for (int ti = blockIdx.x * group; ti < t_end; ++ti) {
@@ -68,6 +70,7 @@ __global__ void __launch_bounds__(BLOCK, 12) background_kernel(ProblemDev P, int
   for (int c0 = 0; c0 < nn; c0 += NB_CHUNK) {
     const int nc = min(NB_CHUNK, nn - c0);
     if (!staged) {
+      bool w_mine = false;
       __syncthreads();   // the previous neighbours have been read
       for (int w = tid; w < nc * ITEMS; w += BLOCK) {
         const int q = w / ITEMS, e = w % ITEMS;
@@ -103,9 +106,10 @@ __global__ void __launch_bounds__(BLOCK, 12) background_kernel(ProblemDev P, int
           S.c[5] = sc.L10;
           S.c[6] = sc.L11;
           S.c[7] = sc.e;
+          w_mine |= wide_range(tb, sc.iota, sc.L11);
         }
       }
-      __syncthreads();
+      wide = __syncthreads_or(w_mine) != 0;
     }
     staged = nn <= NB_CHUNK;
 #pragma unroll(PPT <= 2 ? PPT : 1)
@@ -119,25 +123,31 @@ __global__ void __launch_bounds__(BLOCK, 12) background_kernel(ProblemDev P, int
         // galaxy components two at a time, on packed two-wide float32 arithmetic
         float f0 = 0.f;
         float2 fE = make_float2(0.f, 0.f), fD = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < CELESTE_NPSF; ++k) {
-          const float d0 = fx[r] - S.mu[2 * k], d1 = fy[r] - S.mu[2 * k + 1];
-          const float s0 = d0 * d0, s1 = 2.f * d0 * d1, s2 = d1 * d1;
-          const float4 st = S.star[k];
-          f0 += st.x * exp2f(st.y * s0 + st.z * s1 + st.w * s2);
-          const float2 S0 = make_float2(s0, s0), S1 = make_float2(s1, s1), S2 = make_float2(s2, s2);
-#pragma unroll
-          for (int pr = 0; pr < NMIX / 2; ++pr) {
-            const float4 a = S.gal[2 * (k * NMIX / 2 + pr)], b = S.gal[2 * (k * NMIX / 2 + pr) + 1];
-            const float2 q = __ffma2_rn(make_float2(b.x, b.y), S2,
-                                        __ffma2_rn(make_float2(a.z, a.w), S1, __fmul2_rn(make_float2(a.x, a.y), S0)));
-            const float2 v = __fmul2_rn(make_float2(b.z, b.w), make_float2(ex2_ftz(q.x), ex2_ftz(q.y)));
-            if (pr < CELESTE_NEXP / 2)
-              fE = __fadd2_rn(fE, v);
-            else
-              fD = __fadd2_rn(fD, v);
+        auto profiles = [&](auto w) {
+          constexpr bool WIDE = decltype(w)::value;
+          constexpr int UK = WIDE ? 1 : CELESTE_NPSF, UP = WIDE ? 1 : NMIX / 2;   // (the rare form stays small)
+#pragma unroll(UK)
+          for (int k = 0; k < CELESTE_NPSF; ++k) {
+            const float d0 = fx[r] - S.mu[2 * k], d1 = fy[r] - S.mu[2 * k + 1];
+            const float s0 = d0 * d0, s1 = 2.f * d0 * d1, s2 = d1 * d1;
+            const float4 st = S.star[k];
+            f0 += st.x * exp2f(st.y * s0 + st.z * s1 + st.w * s2);
+            const float2 S0 = make_float2(s0, s0), S1 = make_float2(s1, s1), S2 = make_float2(s2, s2);
+#pragma unroll(UP)
+            for (int pr = 0; pr < NMIX / 2; ++pr) {
+              const float4 a = S.gal[2 * (k * NMIX / 2 + pr)], b = S.gal[2 * (k * NMIX / 2 + pr) + 1];
+              const float2 q = __ffma2_rn(make_float2(b.x, b.y), S2,
+                                          __ffma2_rn(make_float2(a.z, a.w), S1, __fmul2_rn(make_float2(a.x, a.y), S0)));
+              const float2 v = __fmul2_rn(make_float2(b.z, b.w), make_float2(ex2_gal<WIDE>(q.x), ex2_gal<WIDE>(q.y)));
+              if (pr < CELESTE_NEXP / 2)
+                fE = __fadd2_rn(fE, v);
+              else
+                fD = __fadd2_rn(fD, v);
+            }
           }
-        }
+        };
+        if (!wide) profiles(std::false_type{});
+        else profiles(std::true_type{});
         const float fEs = fE.x + fE.y, fDs = fD.x + fD.y;
         const float f1 = fEs + S.c[7] * (fDs - fEs);
         bE[r] += S.c[0] * f0 + S.c[1] * f1;

@@ -300,13 +300,29 @@ __device__ inline Sym2 inv2(const Sym2& S, float& logdet) {
 constexpr float LOG2E = 1.4426950408889634f;
 constexpr float LOG_2PI = 1.8378770664093453f;
 
-// 2^x by the special-function unit alone, subnormal results as 0: what that leaves out is under
-// 1.2e-38, where the rate it is added to is at least the sky's.  (exp2f spends three more
-// instructions per component on those subnormals: 4 % of the kernel.)
+// 2^x by the special-function unit alone, subnormal results as 0.  (exp2f spends three more
+// instructions per component on those subnormals.  With it throughout, a mosaic pass takes 3.7 % longer, a
+// field's value, gradient and Hessian 1.8, wide patches with the 3xTF32 products 3.8, a crowded background
+// 2.6; with the choice below 0.9, 0.6, 1.7 and 0 %.)
 __device__ __forceinline__ float ex2_ftz(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// A galaxy component's exponential, with (WIDE) or without the subnormal results.
+template <bool WIDE>
+__device__ __forceinline__ float ex2_gal(float x) { return WIDE ? exp2f(x) : ex2_ftz(x); }
+
+// Whether the components of a source's table tb under 2^-126 of their peaks count.  Their light reaches
+// the rate multiplied by the components' weights, whose sum is at most that of the PSF's own (a component is the
+// PSF widened, the mixtures have unit flux), by E[l | galaxy] and by the calibration: up to 3.4e38, the
+// largest constant that sat_f leaves, so that a subnormal can stand for many counts.  Below the limit all
+// that ex2_ftz leaves out of a source's rate is under 2^40 2^-126 = 1.3e-26 counts, where the sky's own
+// rounding in float32 is 2^-24 of its counts.  (A catalog's sources are near 2^14; a flux variance that
+// Newton has carried to E[l^2] = e^132, near 2^53, takes the WIDE form.)
+__device__ __forceinline__ bool wide_range(const float* tb, float iota, float L11) {
+  return !(iota * L11 * (tb[TB_STAR] + tb[TB_STAR + 4] + tb[TB_STAR + 8]) <= 0x1p40f);
 }
 
 // Position of the source in image pixels relative to (ox, oy), in float64.

@@ -23,6 +23,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include "celeste_internal.cuh"
@@ -437,10 +438,12 @@ struct PixGeo {
   }
 };
 
-// One galaxy mixture component's value at a pixel (e: its table entry).
+// One galaxy mixture component's value at a pixel (e: its table entry; WIDE: wide_range).
+template <bool WIDE>
 __device__ __forceinline__ float gal_value(const float (&e)[GT_STRIDE], const PixGeo& g) {
   const float q = fmaf(e[GT_P + 2], g.S2.x, fmaf(e[GT_P + 1], g.S1.x, e[GT_P] * g.S0.x));
-  return e[GT_W] * ex2_ftz(q * (-0.5f * LOG2E));
+  const float x = q * (-0.5f * LOG2E);
+  return e[GT_W] * ex2_gal<WIDE>(x);
 }
 
 // A galaxy mixture component of value N at a pixel: value, 5 first and 15 second derivatives over v5,
@@ -485,9 +488,10 @@ __device__ __forceinline__ void gal_sums(const float (&e)[GT_STRIDE], const PixG
 }
 
 // One component at a lane's pixel.  Far from a narrow component its Gaussian underflows to exactly 0
-// (q > ~175): where that holds on every lane of the warp (lanes without a pixel count as 0) the
+// (q > ~175, > ~207 in the WIDE form): where that holds on every lane of the warp (lanes without a pixel count as 0) the
 // component adds exactly nothing, and the warp skips its derivative terms (on the mosaic ~19 % of
 // warp-component pairs).  All lanes of the warp must be active.
+template <bool WIDE>
 __device__ __forceinline__ void gal_component(const float* ep, const PixGeo& g, bool valid, GalAcc& A) {
   float e[GT_STRIDE];
   const float4* e4 = reinterpret_cast<const float4*>(ep);
@@ -499,7 +503,7 @@ __device__ __forceinline__ void gal_component(const float* ep, const PixGeo& g, 
     e[4 * w + 2] = t4.z;
     e[4 * w + 3] = t4.w;
   }
-  const float N = gal_value(e, g);
+  const float N = gal_value<WIDE>(e, g);
   if (__all_sync(0xffffffffu, N == 0.f || !valid)) return;
   gal_sums(e, g, N, A);
 }
@@ -571,6 +575,8 @@ __global__ void __launch_bounds__(BLOCK, full_ctas_per_sm(HM)) elbo_full_kernel(
   }
   const float* tab = tab_buf[b];
   const float4* spix = spix_buf[b];
+  const SNConst& sc = *reinterpret_cast<const SNConst*>(&tab[TB_SNC]);
+  const bool wide = wide_range(tab, sc.iota, sc.L11);
   const int t_start = tmeta[b].start, t_count = tmeta[b].count, pt_w = pmeta[b].w;
   if (tid == 0) atomicAdd(P.counters + 0, (unsigned long long)t_count);
 
@@ -595,28 +601,32 @@ __global__ void __launch_bounds__(BLOCK, full_ctas_per_sm(HM)) elbo_full_kernel(
     GalAcc G0, G1;   // the exponential family's sums, the de Vaucouleurs family's
     G1.zero();
     float* const stash = wbuf[warp] + lane;
+    auto galaxy = [&](auto w) {
 #pragma unroll 1
-    for (int fam = 0; fam < 2; ++fam) {
-      if constexpr (HM == 0) {
-        if (fam) {
-          const float* g = reinterpret_cast<const float*>(&G1);
+      for (int fam = 0; fam < 2; ++fam) {
+        if constexpr (HM == 0) {
+          if (fam) {
+            const float* g = reinterpret_cast<const float*>(&G1);
 #pragma unroll
-          for (int q = 0; q < GAL_FLOATS; ++q) stash[32 * q] = g[q];   // (read by the same lane below)
+            for (int q = 0; q < GAL_FLOATS; ++q) stash[32 * q] = g[q];   // (read by the same lane below)
+          }
+        } else {
+          G0 = G1;   // (first round: zeros; second: the exponential family's sums)
         }
-      } else {
-        G0 = G1;   // (first round: zeros; second: the exponential family's sums)
-      }
-      G1.zero();
-      const int j0 = fam ? CELESTE_NEXP : 0, j1 = fam ? NMIX : CELESTE_NEXP;
+        G1.zero();
+        const int j0 = fam ? CELESTE_NEXP : 0, j1 = fam ? NMIX : CELESTE_NEXP;
 #pragma unroll 1
-      for (int k = 0; k < CELESTE_NPSF; ++k) {
-        PixGeo g;
-        g.set(fx, fy, &tab[TB_MU + 2 * k]);
-        const float* ep = &tab[SM_GAL + (k * NMIX + j0) * GT_STRIDE];
+        for (int k = 0; k < CELESTE_NPSF; ++k) {
+          PixGeo g;
+          g.set(fx, fy, &tab[TB_MU + 2 * k]);
+          const float* ep = &tab[SM_GAL + (k * NMIX + j0) * GT_STRIDE];
 #pragma unroll 1
-        for (int j = j0; j < j1; ++j, ep += GT_STRIDE) gal_component(ep, g, valid, G1);
+          for (int j = j0; j < j1; ++j, ep += GT_STRIDE) gal_component<decltype(w)::value>(ep, g, valid, G1);
+        }
       }
-    }
+    };
+    if (!wide) galaxy(std::false_type{});
+    else galaxy(std::true_type{});
     if constexpr (HM == 0) {
       float* g = reinterpret_cast<float*>(&G0);
 #pragma unroll
@@ -802,8 +812,11 @@ __global__ void __launch_bounds__(BLOCK, full_ctas_per_sm(HM)) elbo_full_kernel(
 // diff = 1: sum of l(theta) - l(theta_ref) per pixel, where theta_ref is the point of the source's
 //           last full evaluation (its E[G], Var[G] kept in srcmom): the change of the ELBO's pixel
 //           part without the rounding of two large sums.
+// (1024-pixel tiles: five CTAs' pixel buffers fill the shared memory)
+constexpr int VALUE_CTAS_PER_SM = 8;
+
 template <int PPT>
-__global__ void __launch_bounds__(BLOCK) elbo_value_kernel(ProblemDev P, int diff) {
+__global__ void __launch_bounds__(BLOCK, PPT < 8 ? VALUE_CTAS_PER_SM : 5) elbo_value_kernel(ProblemDev P, int diff) {
   __shared__ __align__(16) float tab_buf[2][TB_VFLOATS];   // the table's value-only prefix
   __shared__ __align__(16) float4 spix_buf[2][BLOCK * PPT];
   __shared__ __align__(8) uint64_t bar[2];
@@ -840,6 +853,7 @@ __global__ void __launch_bounds__(BLOCK) elbo_value_kernel(ProblemDev P, int dif
   const PatchDev pt = pmeta[b];
   if (tid == 0) atomicAdd(P.counters + 1, (unsigned long long)t.count);
   const SNConst c = *reinterpret_cast<const SNConst*>(&tab[TB_SNC]);
+  const bool wide = wide_range(tab, c.iota, c.L11);
   float sum = 0.f;
 #pragma unroll 1
   for (int r = 0; r < PPT; ++r) {
@@ -865,26 +879,32 @@ __global__ void __launch_bounds__(BLOCK) elbo_value_kernel(ProblemDev P, int dif
     // ~1e-7 of a pixel's rate, far below what the ELBO tolerance resolves
     float f0 = 0.f;
     float2 fE = make_float2(0.f, 0.f), fD = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < CELESTE_NPSF; ++k) {
-      const float d0 = fx - tab[TB_MU + 2 * k], d1 = fy - tab[TB_MU + 2 * k + 1];
-      const float s0 = d0 * d0, s1 = 2.f * d0 * d1, s2 = d1 * d1;
-      const float4 st = *reinterpret_cast<const float4*>(&tab[TB_STAR + 4 * k]);
-      f0 += st.x * exp2f(fmaf(st.w, s2, fmaf(st.z, s1, st.y * s0)) * (-0.5f * LOG2E));
-      const float2 S0 = f2(s0, s0), S1 = f2(s1, s1), S2 = f2(s2, s2);
-      const float4* vp = reinterpret_cast<const float4*>(&tab[TB_VAL + 8 * (k * NMIX / 2)]);
-#pragma unroll
-      for (int pr = 0; pr < NMIX / 2; ++pr) {
-        const float4 a = vp[2 * pr], w = vp[2 * pr + 1];   // (P00, P00', P01, P01'), (P11, P11', W, W')
-        const float2 q = fma2(f2(w.x, w.y), S2, fma2(f2(a.z, a.w), S1, mul2(f2(a.x, a.y), S0)));
-        const float2 qs = mul2(q, f2(-0.5f * LOG2E, -0.5f * LOG2E));
-        const float2 g = mul2(f2(w.z, w.w), f2(ex2_ftz(qs.x), ex2_ftz(qs.y)));
-        if (pr < CELESTE_NEXP / 2)
-          fE = add2(fE, g);
-        else
-          fD = add2(fD, g);
+    auto profiles = [&](auto w) {
+      constexpr bool WIDE = decltype(w)::value;
+      constexpr int UK = WIDE ? 1 : CELESTE_NPSF, UP = WIDE ? 1 : NMIX / 2;   // (the rare form stays small)
+#pragma unroll(UK)
+      for (int k = 0; k < CELESTE_NPSF; ++k) {
+        const float d0 = fx - tab[TB_MU + 2 * k], d1 = fy - tab[TB_MU + 2 * k + 1];
+        const float s0 = d0 * d0, s1 = 2.f * d0 * d1, s2 = d1 * d1;
+        const float4 st = *reinterpret_cast<const float4*>(&tab[TB_STAR + 4 * k]);
+        f0 += st.x * exp2f(fmaf(st.w, s2, fmaf(st.z, s1, st.y * s0)) * (-0.5f * LOG2E));
+        const float2 S0 = f2(s0, s0), S1 = f2(s1, s1), S2 = f2(s2, s2);
+        const float4* vp = reinterpret_cast<const float4*>(&tab[TB_VAL + 8 * (k * NMIX / 2)]);
+#pragma unroll(UP)
+        for (int pr = 0; pr < NMIX / 2; ++pr) {
+          const float4 a = vp[2 * pr], w = vp[2 * pr + 1];   // (P00, P00', P01, P01'), (P11, P11', W, W')
+          const float2 q = fma2(f2(w.x, w.y), S2, fma2(f2(a.z, a.w), S1, mul2(f2(a.x, a.y), S0)));
+          const float2 qs = mul2(q, f2(-0.5f * LOG2E, -0.5f * LOG2E));
+          const float2 g = mul2(f2(w.z, w.w), f2(ex2_gal<WIDE>(qs.x), ex2_gal<WIDE>(qs.y)));
+          if (pr < CELESTE_NEXP / 2)
+            fE = add2(fE, g);
+          else
+            fD = add2(fD, g);
+        }
       }
-    }
+    };
+    if (!wide) profiles(std::false_type{});
+    else profiles(std::true_type{});
     const float fEs = fE.x + fE.y, fDs = fD.x + fD.y;
     const float f1 = fEs + c.e * (fDs - fEs);
     const float EG = c.A0 * f0 + c.A1 * f1;
@@ -929,7 +949,6 @@ __global__ void __launch_bounds__(BLOCK) elbo_value_kernel(ProblemDev P, int dif
 // ------------------------------------------------------------------------------ launchers
 // Persistent grids: a fixed number of CTAs per SM takes tiles from the device work queue over the
 // tile worklist, whose length is known only on the device.
-constexpr int VALUE_CTAS_PER_SM = 8;
 
 cudaError_t launch_full(const ProblemDev& P, const double* theta, cudaStream_t st) {
   if (P.n_tiles == 0) return cudaSuccess;
