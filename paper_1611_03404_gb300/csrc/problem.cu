@@ -101,19 +101,19 @@ __global__ void kappa_kernel(float* kappa) {
   if (i < KAPPA_TABLE) kappa[i] = log_factorial_term((float)i);
 }
 
-// Gather each patch pixel's count and its log-factorial term, one CTA per patch; the fixed rate and variance
-// are written when the background is rendered, which every evaluation needs first.  Counts are whole numbers
-// unless an image has been calibrated, so their terms come from the table (the same function's values):
-// evaluated per pixel the float64 logarithm and lgamma bound the kernel: 8.79 ms for 61 M mosaic pixels, 4 % of
-// a pass (223 -> 205 ms with the other steps of the same time).
-__global__ void __launch_bounds__(256) gather_pixels_kernel(ProblemDev P) {
+// Gather each patch pixel's count and its log-factorial term, gridDim.y CTAs per patch; the fixed rate and
+// variance are written when the background is rendered, which every evaluation needs first.  Whole counts'
+// terms come from the table (the same function's values): evaluated per pixel the float64 logarithm and
+// lgamma bound the kernel, as they still do for the fractional counts of a calibrated image.
+constexpr int GATHER_THREADS = 128, GATHER_CTAS_PER_SM = 128;
+__global__ void __launch_bounds__(GATHER_THREADS) gather_pixels_kernel(ProblemDev P) {
   const PatchDev pt = P.patches[blockIdx.x];
   const ImageDev& im = P.images[pt.image];
   const float* src = im.pixels + (size_t)pt.y0 * im.W + pt.x0;
   const int W = im.W, n = pt.w * pt.h;
   float4* out = P.pix + pt.pix_off;
 #pragma unroll 4
-  for (int i = threadIdx.x; i < n; i += 256) {
+  for (int i = blockIdx.y * GATHER_THREADS + threadIdx.x; i < n; i += gridDim.y * GATHER_THREADS) {
     const int row = i / pt.w, col = i - row * pt.w;
     float x = src[(size_t)row * W + col];
     if (!(x >= 0.f) || !isfinite(x)) {
@@ -280,6 +280,7 @@ void build_layout(celeste_problem* p) {
     a.nbr_end = (int)p->nbr.size();
     a.pix_off = off;
     int npix = a.w * a.h;
+    p->max_patch_pix = std::max(p->max_patch_pix, npix);
     off += npix;
     a.tile_begin = (int)p->tiles.size();
     for (int st = 0; st < npix; st += p->tile_pixels) {
@@ -366,6 +367,18 @@ extern "C" int celeste_problem_counts(const celeste_problem* p, int64_t counts[5
   return CELESTE_OK;
 }
 
+// CTAs per patch: what brings the grid to 128 per SM, at most one per 128 pixels of the largest patch.  One CTA
+// per patch left a fractional count's float64 work to as many SMs as there are patches (refresh of one
+// source's five 129 x 129 patches 381 us, 27 now; whole counts 34 and 15); 16 or 32 per SM leave a tail of
+// large patches (5000 field patches, fractional: 259-263 us, 250 at 128 per SM; whole: 19 and 20).
+static cudaError_t launch_gather(const celeste_problem* p, cudaStream_t st) {
+  const ProblemDev& D = p->dev;
+  const int most = (p->max_patch_pix + GATHER_THREADS - 1) / GATHER_THREADS;
+  const int per_patch = std::max(1, std::min(most, GATHER_CTAS_PER_SM * D.n_sm / D.n_patches));
+  gather_pixels_kernel<<<dim3(D.n_patches, per_patch), GATHER_THREADS, 0, st>>>(D);
+  return cudaGetLastError();
+}
+
 template <class T>
 static cudaError_t upload(char* base, size_t off, const std::vector<T>& v, cudaStream_t st) {
   if (v.empty()) return cudaSuccess;
@@ -446,8 +459,7 @@ extern "C" int celeste_problem_bind(celeste_problem* p, void* workspace, size_t 
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "psf_setup_kernel");
     kappa_kernel<<<KAPPA_TABLE / 64, 64, 0, st>>>(reinterpret_cast<float*>(base + L.kappa));
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kappa_kernel");
-    gather_pixels_kernel<<<D.n_patches, 256, 0, st>>>(D);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "gather_pixels_kernel");
+    if ((e = launch_gather(p, st)) != cudaSuccess) return cuda_fail(e, "gather_pixels_kernel");
   }
   p->bound = true;
   p->background_ready = false;
@@ -462,8 +474,7 @@ extern "C" int celeste_problem_refresh_pixels(celeste_problem* p, celeste_stream
   cudaError_t e = cudaMemsetAsync(D.err, 0, sizeof(int) * 4, st);
   if (e != cudaSuccess) return cuda_fail(e, "clear err");
   if (D.n_patches > 0) {
-    gather_pixels_kernel<<<D.n_patches, 256, 0, st>>>(D);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "gather_pixels_kernel");
+    if ((e = launch_gather(p, st)) != cudaSuccess) return cuda_fail(e, "gather_pixels_kernel");
   }
   p->background_ready = false;
   return CELESTE_OK;

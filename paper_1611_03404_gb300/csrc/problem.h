@@ -42,6 +42,7 @@ struct celeste_problem {
   std::vector<celeste::ImageDev> imgdev;
   std::vector<double> psf_coef;
   long long n_pix = 0;
+  int max_patch_pix = 0;                              // pixels of the largest patch
   celeste::WsLayout ws{};
   // binding
   char* base = nullptr;
