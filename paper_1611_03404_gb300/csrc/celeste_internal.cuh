@@ -105,7 +105,7 @@ constexpr int WL_INTS = 8;
 constexpr int TR_CACHE = NP * NP + 5 * NP;
 // Doubles of the multiplier searches' factor tables (one per problem).
 constexpr int TR_FACTORS = 640;
-// Whole counts whose log-factorial term is tabulated (256 KB; larger ones are evaluated).
+// Whole counts whose log-factorial term is tabulated, at most (256 KB; larger ones are evaluated).
 constexpr int KAPPA_TABLE = 65536;
 
 // Device view of a bound problem (passed by value to kernels).
@@ -119,7 +119,8 @@ struct ProblemDev {
   const double* psf_coef;        // [n_images][3][6][6]
   float* psf;                    // [n_patches][18]: per PSF comp (w, mx, my, s00, s01, s11)
   float4* pix;                   // [n_pix]: (x, fixed rate, fixed variance, log-factorial term)
-  const float* kappa;            // [KAPPA_TABLE] log-factorial term of the whole counts
+  const float* kappa;            // [n_kappa] log-factorial term of the whole counts
+  int n_kappa;                   // as many as there are patch pixels, at most KAPPA_TABLE
   float2* srcmom;                // [n_pix]: the target source's (E[G], Var[G]) at its last full evaluation
   float* ptab;                   // [n_patches][TB_FLOATS] per-patch tables
   const long long* tile_pix;     // [n_tiles] the tile's first float4 in pix (patch offset + start)

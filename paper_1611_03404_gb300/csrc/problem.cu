@@ -95,10 +95,10 @@ __device__ inline float log_factorial_term(float x) {
   return (float)(xd > 0 ? xd * log(xd) - xd - lgamma(xd + 1.0) : 0.0);
 }
 
-// The term of the whole counts 0 .. KAPPA_TABLE - 1, once per bind.
-__global__ void kappa_kernel(float* kappa) {
+// The term of the whole counts 0 .. n - 1, once per bind.
+__global__ void kappa_kernel(float* kappa, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < KAPPA_TABLE) kappa[i] = log_factorial_term((float)i);
+  if (i < n) kappa[i] = log_factorial_term((float)i);
 }
 
 // Gather each patch pixel's count and its log-factorial term, gridDim.y CTAs per patch; the fixed rate and
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) gather_pixels_kernel(ProblemDe
       atomicExch(P.err + ERR_BAD_PIXEL, 1);
       x = 0.f;
     }
-    const float kappa = x < (float)KAPPA_TABLE && x == truncf(x) ? P.kappa[(int)x] : log_factorial_term(x);
+    const float kappa = x < (float)P.n_kappa && x == truncf(x) ? P.kappa[(int)x] : log_factorial_term(x);
     out[i] = make_float4(x, 0.f, 0.f, kappa);
   }
 }
@@ -213,6 +213,10 @@ extern "C" int celeste_problem_create(const celeste_problem_desc* d, celeste_pro
 }
 
 namespace celeste {
+
+// Entries of the log-factorial table: no more than the patches have pixels, so that filling it is never more
+// float64 work than the first gather without it.
+int kappa_entries(const celeste_problem* p) { return (int)std::min<long long>(KAPPA_TABLE, p->n_pix); }
 
 void build_layout(celeste_problem* p) {
   const int S = p->S, N = (int)p->images.size();
@@ -349,7 +353,7 @@ void build_layout(celeste_problem* p) {
   L.nt_lam = take(sizeof(double) * S);
   L.nt_list = take(sizeof(int) * S);
   L.nt_fac = take(sizeof(double) * TR_FACTORS);
-  L.kappa = take(sizeof(float) * KAPPA_TABLE);
+  L.kappa = take(sizeof(float) * kappa_entries(p));
   L.total = o;
 }
 
@@ -434,6 +438,7 @@ extern "C" int celeste_problem_bind(celeste_problem* p, void* workspace, size_t 
   D.wl_count = reinterpret_cast<int*>(base + L.wl_count);
   D.snc = reinterpret_cast<SNConst*>(base + L.snc);
   D.kappa = reinterpret_cast<const float*>(base + L.kappa);
+  D.n_kappa = kappa_entries(p);
   D.pweight = nullptr;   // set only on the joint solver's copies
   D.refEV = nullptr;
   D.n_sm = std::max(n_sm, 1);
@@ -457,7 +462,7 @@ extern "C" int celeste_problem_bind(celeste_problem* p, void* workspace, size_t 
   if (D.n_patches > 0) {
     psf_setup_kernel<<<(D.n_patches + 127) / 128, 128, 0, st>>>(D);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "psf_setup_kernel");
-    kappa_kernel<<<KAPPA_TABLE / 64, 64, 0, st>>>(reinterpret_cast<float*>(base + L.kappa));
+    kappa_kernel<<<(D.n_kappa + 63) / 64, 64, 0, st>>>(reinterpret_cast<float*>(base + L.kappa), D.n_kappa);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kappa_kernel");
     if ((e = launch_gather(p, st)) != cudaSuccess) return cuda_fail(e, "gather_pixels_kernel");
   }
