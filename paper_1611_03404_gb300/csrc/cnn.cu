@@ -854,6 +854,8 @@ extern "C" int celeste_cnn_forward_budget(const float* params, const uint16_t* p
   if ((out_scale == nullptr) != (out_shift == nullptr)) return fail(CELESTE_ERR_INVALID_ARG, "scale and shift go together");
   if (engine != CELESTE_CNN_MMA_SYNC && engine != CELESTE_CNN_TCGEN05)
     return fail(CELESTE_ERR_INVALID_ARG, "engine must be CELESTE_CNN_MMA_SYNC or CELESTE_CNN_TCGEN05");
+  if (engine == CELESTE_CNN_TCGEN05 && reinterpret_cast<uintptr_t>(params_bf16) % 16)
+    return fail(CELESTE_ERR_INVALID_ARG, "params_bf16 must be 16-byte aligned (it is copied 16 bytes at a time)");
   int rc = check_ws(batch, ws, ws_bytes);
   if (rc != CELESTE_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
