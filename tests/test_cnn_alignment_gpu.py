@@ -18,8 +18,8 @@ def test_backward_with_shifted_weights(batch, shift):
     from paper_1611_03404_gb300 import cnn
     dev = torch.device("cuda:0")
     gen = torch.Generator(device=dev).manual_seed(batch)
-    x = torch.randn(batch, 32, 32, 5, device=dev, generator=gen).to(torch.bfloat16).view(torch.int16)
-    dy = torch.randn(batch, 27, device=dev, generator=gen)
+    x = torch.randn(batch, 32, 32, 5, device=dev, dtype=torch.float32, generator=gen).to(torch.bfloat16).view(torch.int16)
+    dy = torch.randn(batch, 27, device=dev, dtype=torch.float32, generator=gen)
     net = cnn.WarmStartCNN(dev, seed=6)
     net.forward(x)
     net.grad.zero_()

@@ -22,7 +22,7 @@ def test_waits_that_run_out(batch, budget):
     dev = torch.device("cuda:0")
     net = cnn.WarmStartCNN(dev, seed=6)
     gen = torch.Generator(device=dev).manual_seed(batch)
-    x = torch.randn(batch, 32, 32, 5, device=dev, generator=gen).to(torch.bfloat16).view(torch.int16)
+    x = torch.randn(batch, 32, 32, 5, device=dev, dtype=torch.float32, generator=gen).to(torch.bfloat16).view(torch.int16)
     ref = net.forward(x)
     assert P.lib().celeste_cnn_status() == 0
     _, ws, nb = net.workspace(batch)
