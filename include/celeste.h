@@ -435,7 +435,8 @@ int celeste_cnn_forward(const float* params, const uint16_t* params_bf16, const 
  *     operands gathered into 128-byte-swizzled shared memory, tcgen05.mma into a tensor-memory
  *     accumulator, tcgen05.ld epilogue (bias, ReLU).  Waits are bounded: a product that does not
  *     complete sets an error word that celeste_cnn_status reports.
- * Both use BF16 operands and FP32 accumulation; their outputs differ only in summation order. */
+ * Both use BF16 operands and FP32 accumulation, and add a sum's products in the same order: the tests hold
+ * their outputs to the same bits. */
 enum { CELESTE_CNN_MMA_SYNC = 0, CELESTE_CNN_TCGEN05 = 1 };
 int celeste_cnn_forward_ex(const float* params, const uint16_t* params_bf16, const uint16_t* x, int batch,
                            const float* out_scale, const float* out_shift, float* y, void* ws, size_t ws_bytes,
