@@ -519,9 +519,9 @@ __device__ __forceinline__ void gal_component(const float* ep, const PixGeo& g, 
 // in registers; the FP32 form keeps the other's in the warp's transpose scratch until the pixel's term,
 // and so fits 96 registers and 5 CTAs of four warps per SM (before: both families' sums live, 125
 // registers, 4 CTAs).  What bounds it then is the register file: a packed FMA on three distinct register
-// pairs issues every 3.4 cycles (two scalar ones every 2.2, but they take two slots: all-scalar and
-// mixed forms ran 1-8 % slower; two pixels per lane at 168 registers: 1 % slower, and a tile takes 4 us
-// longer).  13.5 M mosaic pixels, one value + gradient + Hessian call: 2.53 -> 2.34 ms (256-pixel tiles
+// pairs issues every 3.0 cycles of a sub-partition, where one that keeps two of them takes 2.2 (the two scalar
+// FMAs in its place: 3.1 and 2.1, in two slots; all-scalar and mixed forms ran 1-8 % slower; two pixels per lane at
+// 168 registers: 1 % slower, and a tile takes 4 us longer).  13.5 M mosaic pixels, one value + gradient + Hessian call: 2.53 -> 2.34 ms (256-pixel tiles
 // 2.88 -> 2.23, 512-pixel 2.59 -> 2.23); a 1000-source field 559 -> 536 us.  The tensor-core forms spill
 // at 96 registers and stay at 4 CTAs (3xTF32: 3.02 -> 2.76 ms; with 5 CTAs 2.78).
 constexpr int SM_GAL = TB_VAL;                              // the galaxy entries' offset in the staged table
