@@ -423,7 +423,7 @@ int celeste_cnn_init(float* params, uint16_t* params_bf16, uint64_t seed, celest
 /* y [batch][27] = network(x [batch][32][32][5]); with out_scale / out_shift (both or neither,
  * [27]) the output is y * scale + shift.  Keeps the activations in ws for celeste_cnn_backward.
  * params_bf16 must be 16-byte aligned (CELESTE_ERR_INVALID_ARG otherwise; celeste_cnn_backward and the
- * mma.sync engine take it anywhere), x may start anywhere.
+ * mma.sync engine take it anywhere), x may start anywhere; at most 2097151 patches (CELESTE_ERR_INVALID_ARG).
  * Runs on the tcgen05 tensor cores (celeste_cnn_forward_ex with CELESTE_CNN_TCGEN05). */
 int celeste_cnn_forward(const float* params, const uint16_t* params_bf16, const uint16_t* x, int batch,
                         const float* out_scale, const float* out_shift, float* y, void* ws, size_t ws_bytes,

@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdint>
 
 #include "celeste_internal.cuh"
@@ -856,6 +857,8 @@ extern "C" int celeste_cnn_forward_budget(const float* params, const uint16_t* p
     return fail(CELESTE_ERR_INVALID_ARG, "engine must be CELESTE_CNN_MMA_SYNC or CELESTE_CNN_TCGEN05");
   if (engine == CELESTE_CNN_TCGEN05 && reinterpret_cast<uintptr_t>(params_bf16) % 16)
     return fail(CELESTE_ERR_INVALID_ARG, "params_bf16 must be 16-byte aligned (it is copied 16 bytes at a time)");
+  if (batch > INT_MAX / (IMG * IMG))   // (the first layer's rows, one per pixel, are an int)
+    return fail(CELESTE_ERR_INVALID_ARG, "batch must be at most %d", INT_MAX / (IMG * IMG));
   int rc = check_ws(batch, ws, ws_bytes);
   if (rc != CELESTE_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
